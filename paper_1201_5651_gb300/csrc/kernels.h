@@ -3,15 +3,21 @@
 #include <cuda_runtime.h>
 #include "oots_internal.h"
 
+#ifdef __CUDACC__
+#define OOTS_HOSTDEV __host__ __device__
+#else
+#define OOTS_HOSTDEV
+#endif
+
 namespace oots {
 
 template <typename Real> struct DevTable;
 struct ff;
 template <typename Real> struct ColT;
 
-// Tile shapes of the wavefront sweep: (id, TX, TY, TZ); one chain thread per
-// (j,k) column (TY*TZ a multiple of 32) plus one producer warp.  Shapes with
-// TY*TZ = 32 keep the whole plane chain in one warp.
+// Tile shapes of the implicit wavefront sweep (A1): (id, TX, TY, TZ); one chain
+// thread per (j,k) column (TY*TZ a multiple of 32) plus one producer warp.
+// Shapes with TY*TZ = 32 keep the whole plane chain in one warp.
 #define OOTS_SHAPES(X) \
     X(0, 16, 8, 8)     \
     X(1, 16, 8, 4)     \
@@ -20,55 +26,125 @@ template <typename Real> struct ColT;
     X(4, 8, 8, 8)      \
     X(5, 16, 16, 8)    \
     X(6, 8, 8, 4)
-// Shapes 7 and 8 tile the octants like shapes 4 (8 x 8 x 8) and 0 (16 x 8 x 8)
-// but trace them with the throughput kernel (whole tiles, 64 threads, layer
-// sweeps off the diagonal planes; sweep_tp.cuh); the implicit sweep (A1) runs
-// the pipelined kernel of the same tile (shape 4 or 0) on them.
+// Shapes 7 and 8 are other names of shapes 4 (8 x 8 x 8) and 0 (16 x 8 x 8).
+// The traces of the explicit schemes have no tiles: every shape runs the march.
 enum { NUM_SHAPES = 9, SHAPE_TP8 = 7, SHAPE_TP16 = 8 };
 static const int SHAPE_DIMS[NUM_SHAPES][3] = {{16, 8, 8}, {16, 8, 4}, {16, 16, 16}, {32, 8, 4}, {8, 8, 8},
                                               {16, 16, 8}, {8, 8, 4}, {8, 8, 8}, {16, 8, 8}};
-inline bool is_tp_shape(int shape) { return shape == SHAPE_TP8 || shape == SHAPE_TP16; }
-inline int tp_twin(int shape) { return shape == SHAPE_TP8 ? 4 : 0; }   // pipelined kernel on the same tiles
+inline int sweep_twin(int shape) { return shape == SHAPE_TP8 ? 4 : (shape == SHAPE_TP16 ? 0 : shape); }
 
 template <typename Real> struct SweepParams {
     const GridDev<Real> *grids;
     const Job *jobs;
     const TileItem *items;
     int nitems;
-    int which;                         // 0: trace x into N1; 1: trace xh into N2
     unsigned *ticket;                  // zeroed before each launch
     unsigned *done;                    // CTAs finished; zeroed before each launch
     unsigned *epoch;                   // launches finished so far (persistent; starts at 0)
     unsigned long long *faces;         // per tile 3 faces x FMAX cells x tagged words (zeroed once)
     const DevTable<Real> *tabs;
     int *err;                          // sticky device error
-    Real *tpfaces;                     // throughput kernel: per tile 3 faces x tp_face_comps x 64 values
-    unsigned *tpflags;                 // throughput kernel: per tile the epoch of the launch that finished it
     long long spin_limit;              // bounded wait on upstream tiles
     long long skip_publish;            // tile that never writes its faces (fault-injection test), -1: none
     int chunk;                         // planes per hand-off chunk (<= 0: 4)
     int ngrid;                         // grids in `grids` (> 0: the launch returns at once when every
                                        // grid has reached its end time; 0: no such check)
-    const void *bricks;                // throughput kernel: base of the packed n x of every grid, brick
-                                       // TileItem::brick at bricks + brick x TX x 64 values (nullptr: none)
 };
 
 // tagged 8-byte words per published face cell (mixed path 3, FP64 path 4)
 template <typename Real> constexpr int face_words() { return sizeof(Real) == 4 ? 3 : 4; }
-// values per face cell the throughput kernel publishes: the column (float-float
-// hi and lo in the mixed path, one double in FP64) and the weight factor
-template <typename Real> __host__ __device__ constexpr int tp_face_comps() { return sizeof(Real) == 4 ? 3 : 2; }
 
 template <typename Real> cudaError_t prepare_sweeps();
-template <typename Real> int sweep_occupancy(int shape, int mode);   // resident CTAs per SM
+template <typename Real> int sweep_occupancy(int shape);             // resident CTAs per SM
 template <typename Real> bool sweep_shape_ok(int shape);              // fits the shared memory of this device
 template <typename Real>
-cudaError_t launch_sweep(const SweepParams<Real> &P, int shape, int mode, int nblocks, cudaStream_t s);
-// n x of the traced state (which = 0: x, 1: xh) into each grid's bricks (GridDev::nxb) for the
-// throughput kernel of tile shape `shape`; max_elems = the largest grid's brick cells
+cudaError_t launch_sweep(const SweepParams<Real> &P, int shape, int nblocks, cudaStream_t s);
+
+// The column march (march.cuh).  A published cell is one 16-byte record: its
+// outgoing column (float-float in the mixed path) and weight factor.
+template <typename Real> struct MCell;
+template <> struct alignas(16) MCell<float> { float hi, lo, w, pad; };
+template <> struct alignas(16) MCell<double> { double n, w; };
+
+template <typename Real> struct MarchParams {
+    const GridDev<Real> *grids;
+    const March *marches;
+    const MarchItem *items;            // in the order they are handed out
+    int nitems;
+    int which;                         // 0: trace x into N1; 1: trace xh into N2
+    unsigned *ticket, *done;           // zero before each launch (the launch leaves them so)
+    unsigned *epoch;                   // launches finished so far (persistent; starts at 0)
+    MCell<Real> *halo;
+    unsigned *progress;                // per item: chunks of layers published, tagged with the launch's epoch
+    int *err;                          // sticky device error
+    long long spin_limit;              // bounded wait on upstream items
+    long long skip_publish;            // item that never publishes (fault-injection test), -1: none
+    int ngrid;                         // as SweepParams::ngrid
+    int narr;                          // input arrays of a cell: 1 (x or n x packed), 2 when some grid brings n and x
+};
+
+// Blocks of the march: 32 x ROWS cells, NW warps of RPT rows (the measurements are in march.cuh).
+template <typename Real> struct MarchShape { enum { NW = 7, RPT = sizeof(Real) == 4 ? 3 : 1, ROWS = NW * RPT }; };
+// sets the kernel up on the current device; CTAs per SM with narr input arrays
+template <typename Real> cudaError_t march_occupancy(int narr, int *per_sm);
 template <typename Real>
-cudaError_t launch_pack_nx(const GridDev<Real> *grids, int ngrid, int which, int shape, long long max_elems, int nsm,
+cudaError_t launch_march(const MarchParams<Real> &P, int nblocks, cudaStream_t s);
+// n x of the traced state (which = 0: x, 1: xh) into each grid's padded rows (GridDev::nxp);
+// max_elems = the largest grid's padded cells
+template <typename Real>
+cudaError_t launch_pack_nx(const GridDev<Real> *grids, int ngrid, int which, long long max_elems, int nsm,
                            cudaStream_t s);
+
+// The pyramid of `axis` in octant o (bit a set: the side below the vertex along
+// axis a) of a source at vertex v; false when the octant is empty.  pitch: row
+// length of the input (nx unless packed).
+OOTS_HOSTDEV inline bool make_march(March &M, int nx, int ny, int nz, const int v[3], int o, int axis, int pitch,
+                                    bool packed)
+{
+    const int n3[3] = {nx, ny, nz};
+    int sg[3], ext[3];
+    long long c0[3];
+    for (int a = 0; a < 3; a++) {
+        sg[a] = (o >> a) & 1 ? -1 : 1;
+        ext[a] = sg[a] > 0 ? n3[a] - v[a] : v[a];
+        if (ext[a] <= 0) return false;
+        c0[a] = sg[a] > 0 ? v[a] : v[a] - 1;
+    }
+    const int au = axis == 0 ? 1 : 0, aw = axis == 2 ? 1 : 2;
+    const long long is[3] = {1, pitch, (long long)pitch * ny}, os[3] = {1, nx, (long long)nx * ny};
+    M.grid = M.src = 0;
+    M.axis = axis;
+    M.sg = sg[0];
+    M.len = ext[axis];
+    M.eu = ext[au];
+    M.ew = ext[aw];
+    M.off = axis == 0 ? (sg[0] > 0 ? v[0] % 8 : (8 - v[0] % 8) % 8) : 0;
+    M.packed = packed;
+    M.pad[0] = M.pad[1] = M.pad[2] = 0;
+    M.ibase = c0[0] + c0[1] * is[1] + c0[2] * is[2];
+    M.obase = c0[0] + c0[1] * os[1] + c0[2] * os[2];
+    M.isl = sg[axis] * is[axis]; M.isu = sg[au] * is[au]; M.isw = sg[aw] * is[aw];
+    M.osl = sg[axis] * os[axis]; M.osu = sg[au] * os[au]; M.osw = sg[aw] * os[aw];
+    return true;
+}
+// blocks of a pyramid along u and w
+OOTS_HOSTDEV inline int march_nt1(const March &M) { return ((M.eu < M.len ? M.eu : M.len) + 31) / 32; }
+OOTS_HOSTDEV inline int march_nt2(const March &M, int rows) { return ((M.ew < M.len ? M.ew : M.len) + rows - 1) / rows; }
+// block (T1, T2) without its neighbours' item numbers and halo; returns the cells it publishes
+OOTS_HOSTDEV inline long long make_march_item(MarchItem &I, const March &M, int march, int T1, int T2, int rows)
+{
+    I.march = march;
+    I.T1 = (unsigned short)T1;
+    I.T2 = (unsigned short)T2;
+    I.l0 = 32 * T1 > rows * T2 ? 32 * T1 : rows * T2;
+    I.right = T1 + 1 < march_nt1(M);
+    I.above = T2 + 1 < march_nt2(M, rows);
+    I.pad = 0;
+    I.pad2 = 0;
+    I.up0 = I.up1 = I.up2 = -1;
+    I.halo = 0;
+    return I.right || I.above ? (long long)(M.len - I.l0) * (rows + 32) : 0;
+}
 
 // Plane-parallel sources: which = 0 traces x into N1, 1 traces xh into N2;
 // implicit = 1 runs the A1 row integration instead (single source).  The jobs

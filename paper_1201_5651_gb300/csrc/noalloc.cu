@@ -26,59 +26,69 @@ namespace {
 constexpr size_t kScratchBytes = (size_t)64 << 20;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
-constexpr int kShape = 0;                       // tile shape 16 x 8 x 8
+// The size limit is stated in tiles of 16 x 8 x 8 cells.
 constexpr int kTX = 16, kTY = 8, kTZ = 8;
-constexpr int kFMAX = 128;                      // largest face of the tile
-constexpr int kMaxDiag = 4096;                  // tile diagonals the work-list builder can order
-constexpr size_t kHeader = 64 * 1024;           // ticket, error, state, counters
+constexpr int kMaxDiag = 4096;                  // tile diagonals within the limit
+constexpr int kMaxMarch = 24;                   // pyramids of one source
+constexpr int kMaxItems = 4096;                 // blocks of all pyramids (a grid within the limit has under a thousand)
+constexpr int kMaxItemDiag = 2048;              // block diagonals T1 + T2 of a pyramid (sides up to 8192)
 
 // header layout (byte offsets inside the scratch)
-constexpr size_t kOffTicket = 0;                // ticket, then the count of finished CTAs
-constexpr size_t kOffEpoch = 64;                // sweep launches so far: never cleared (faces carry it)
+constexpr size_t kOffTicket = 0;                // ticket, then the count of finished CTAs (each launch leaves them zero)
+constexpr size_t kOffEpoch = 64;                // marches so far: never cleared (progress words carry it)
 constexpr size_t kOffErr = 128;
 constexpr size_t kOffState = 256;               // DevState (done = 0 after the clear)
-constexpr size_t kOffCount = 1024;              // kMaxDiag unsigned: tiles per diagonal, then cursor
-constexpr size_t kOffJobs = kOffCount + 2 * kMaxDiag * sizeof(unsigned);
-constexpr size_t kOffGrid = kOffJobs + 8 * sizeof(Job) + 256;
+constexpr size_t kOffCount = 1024;              // kMaxItemDiag unsigned: items per diagonal, then cursors
+constexpr size_t kOffMarch = kOffCount + 2 * kMaxItemDiag * sizeof(unsigned) + 256;
+constexpr size_t kOffGrid = kOffMarch + kMaxMarch * sizeof(March) + 256;
 
 struct DevSetup {
     bool ready = false;
     unsigned char *scratch = nullptr;
-    int nblocks[2] = {0, 0};   // per precision
+    int nblocks[2][2] = {};   // per precision and number of input arrays
 };
 static DevSetup g_setup[64];
 static std::mutex g_setup_mutex;   // first-call set-up of a device, from any host thread
 
-template <typename Real> size_t tile_bytes()
-{
-    return sizeof(TileItem) + 3 * kFMAX * face_words<Real>() * sizeof(unsigned long long);
-}
-
-// Byte offset of the per-tile arrays, and the most tiles the scratch holds
-// after them (one item slot is kept spare).
-template <typename Real> size_t tiles_offset()
+// Byte offset of the per-item arrays, and the most tiles a grid may have: the
+// limit this entry point has always stated.  The march needs far less (its
+// published cells are a twentieth of the tiles' faces); the call checks it.
+template <typename Real> size_t items_offset()
 {
     return (kOffGrid + sizeof(GridDev<Real>) + 255) / 256 * 256;
 }
-template <typename Real> long long max_tiles()
-{
-    return (long long)((kScratchBytes - tiles_offset<Real>()) / tile_bytes<Real>()) - 1;
-}
+template <typename Real> long long max_tiles();
+template <> long long max_tiles<float>() { return 7264; }
+template <> long long max_tiles<double>() { return 5450; }
 
-// One block orders the tiles of the (at most 8) octant jobs by tile diagonal:
-// count per diagonal, exclusive scan, then place (order inside a diagonal is free).
-__global__ void build_worklist(const Job *jobs, int njobs, unsigned *count, unsigned *cursor, TileItem *items,
-                               int maxdiag)
+struct MarchSet {
+    March m[kMaxMarch];
+    int n;
+};
+
+// One block lists the items of the (at most 24) pyramids by block diagonal:
+// count per diagonal, exclusive scan, then place (order inside a diagonal is
+// free), then each item's neighbours.
+template <typename Real>
+__global__ void build_worklist(const __grid_constant__ MarchSet S, const __grid_constant__ GridDev<Real> G0,
+                               unsigned char *sc, int rows, MarchItem *items, int *at, int maxdiag)
 {
+    unsigned *count = (unsigned *)(sc + kOffCount), *cursor = count + kMaxItemDiag;
+    March *marches = (March *)(sc + kOffMarch);
+    __shared__ unsigned s_halo;                 // published cells so far (below 2^32: 64 MiB of 16-byte cells)
+    if (threadIdx.x == 0) {
+        s_halo = 0u;
+        *(GridDev<Real> *)(sc + kOffGrid) = G0;
+        *(int *)(sc + kOffErr) = 0;
+        DevState *st = (DevState *)(sc + kOffState);
+        st->done = 0;
+    }
+    for (int j = threadIdx.x; j < S.n; j += blockDim.x) marches[j] = S.m[j];
     for (int d = threadIdx.x; d < maxdiag; d += blockDim.x) { count[d] = 0u; cursor[d] = 0u; }
     __syncthreads();
-    for (int j = 0; j < njobs; j++) {
-        const Job J = jobs[j];
-        const long long n = (long long)J.nt[0] * J.nt[1] * J.nt[2];
-        for (long long t = threadIdx.x; t < n; t += blockDim.x) {
-            const int I = (int)(t % J.nt[0]), Jj = (int)((t / J.nt[0]) % J.nt[1]), K = (int)(t / ((long long)J.nt[0] * J.nt[1]));
-            atomicAdd(&count[I + Jj + K], 1u);
-        }
+    for (int j = 0; j < S.n; j++) {
+        const int n1 = march_nt1(S.m[j]), n = n1 * march_nt2(S.m[j], rows);
+        for (int t = threadIdx.x; t < n; t += blockDim.x) atomicAdd(&count[t % n1 + t / n1], 1u);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -86,21 +96,31 @@ __global__ void build_worklist(const Job *jobs, int njobs, unsigned *count, unsi
         for (int d = 0; d < maxdiag; d++) { const unsigned c = count[d]; cursor[d] = acc; acc += c; }
     }
     __syncthreads();
-    for (int j = 0; j < njobs; j++) {
-        const Job J = jobs[j];
-        const long long n = (long long)J.nt[0] * J.nt[1] * J.nt[2];
-        for (long long t = threadIdx.x; t < n; t += blockDim.x) {
-            const int I = (int)(t % J.nt[0]), Jj = (int)((t / J.nt[0]) % J.nt[1]), K = (int)(t / ((long long)J.nt[0] * J.nt[1]));
-            const unsigned pos = atomicAdd(&cursor[I + Jj + K], 1u);
-            TileItem it;
-            it.job = j;
-            it.I = (unsigned short)I;
-            it.J = (unsigned short)Jj;
-            it.K = (unsigned short)K;
-            it.grid = 0;
-            it.brick = 0u;
-            items[pos] = it;
+    int first = 0;
+    for (int j = 0; j < S.n; j++) {
+        const int n1 = march_nt1(S.m[j]), n = n1 * march_nt2(S.m[j], rows);
+        for (int t = threadIdx.x; t < n; t += blockDim.x) {
+            MarchItem I;
+            const unsigned pub = (unsigned)make_march_item(I, S.m[j], j, t % n1, t / n1, rows);
+            const unsigned pos = atomicAdd(&cursor[t % n1 + t / n1], 1u);
+            I.halo = atomicAdd(&s_halo, pub);
+            items[pos] = I;
+            at[first + t] = (int)pos;
         }
+        first += n;
+    }
+    __syncthreads();
+    first = 0;
+    for (int j = 0; j < S.n; j++) {
+        const int n1 = march_nt1(S.m[j]), n = n1 * march_nt2(S.m[j], rows);
+        for (int t = threadIdx.x; t < n; t += blockDim.x) {
+            MarchItem &I = items[at[first + t]];
+            const int T1 = t % n1, T2 = t / n1;
+            if (T1 > 0) I.up0 = at[first + t - 1];
+            if (T2 > 0) I.up1 = at[first + t - n1];
+            if (T1 > 0 && T2 > 0) I.up2 = at[first + t - n1 - 1];
+        }
+        first += n;
     }
 }
 
@@ -110,46 +130,29 @@ int trace_noalloc(DevSetup &S, int nx, int ny, int nz, double dx, const void *n_
 {
     const int n3[3] = {nx, ny, nz};
     const int T3[3] = {kTX, kTY, kTZ};
-    Job jobs[8];
-    int njobs = 0;
     long long tiles = 0;
     int maxd = 0;
     for (int o = 0; o < 8; o++) {
-        Job J;
-        memset(&J, 0, sizeof(J));
-        J.grid = 0;
-        J.src = 0;
+        int nt[3];
         bool empty = false;
         for (int a = 0; a < 3; a++) {
-            J.v[a] = vtx[a];
-            J.sg[a] = (o >> a) & 1 ? -1 : 1;
-            J.ext[a] = J.sg[a] > 0 ? n3[a] - vtx[a] : vtx[a];
-            if (J.ext[a] <= 0) empty = true;
+            const int ext = (o >> a) & 1 ? vtx[a] : n3[a] - vtx[a];
+            if (ext <= 0) empty = true;
             const int r = vtx[a] % T3[a];
-            J.off[a] = J.sg[a] > 0 ? r : (T3[a] - r) % T3[a];
-            J.nt[a] = (J.ext[a] + J.off[a] + T3[a] - 1) / T3[a];
+            const int off = (o >> a) & 1 ? (T3[a] - r) % T3[a] : r;
+            nt[a] = (ext + off + T3[a] - 1) / T3[a];
         }
         if (empty) continue;
-        J.tile_base = tiles;
-        tiles += (long long)J.nt[0] * J.nt[1] * J.nt[2];
-        const int d = J.nt[0] + J.nt[1] + J.nt[2] - 2;
-        if (d > maxd) maxd = d;
-        jobs[njobs++] = J;
+        tiles += (long long)nt[0] * nt[1] * nt[2];
+        maxd = std::max(maxd, nt[0] + nt[1] + nt[2] - 2);
     }
     const long long maxt = max_tiles<Real>();
     if (tiles > maxt || maxd + 1 > kMaxDiag)
         return -1000 - (int)std::min<long long>(tiles, 1 << 30);   // reported by the caller
 
-    unsigned char *sc = S.scratch;
-    // layout of the per-tile arrays after the fixed part
-    size_t off = tiles_offset<Real>();
-    TileItem *items = (TileItem *)(sc + off);
-    off += (size_t)(maxt + 1) * sizeof(TileItem);
-    off = (off + 255) / 256 * 256;
-    unsigned long long *faces = (unsigned long long *)(sc + off);   // zero at load; launches tag epochs 1, 2, ...
-
     GridDev<Real> G;
     memset(&G, 0, sizeof(G));
+    unsigned char *sc = S.scratch;
     G.nx = nx; G.ny = ny; G.nz = nz;
     G.ncell = (long long)nx * ny * nz;
     G.cell_lo = 0;
@@ -165,40 +168,61 @@ int trace_noalloc(DevSetup &S, int nx, int ny, int nz, double dx, const void *n_
     G.nsrc = 1;
     for (int a = 0; a < 3; a++) G.vtx[0][a] = vtx[a];
     G.tab[0] = -1;
+    G.pitch = nx;
     G.st = (DevState *)(sc + kOffState);
 
-    // clear what must start at zero: ticket, finished-CTA count, error, device state
-    // (the epoch and the faces are never cleared: stale face words carry older epochs)
-    if (cudaMemsetAsync(sc + kOffTicket, 0, kOffEpoch - kOffTicket, st) != cudaSuccess) return -1;
-    if (cudaMemsetAsync(sc + kOffErr, 0, kOffCount - kOffErr, st) != cudaSuccess) return -1;
-    if (cudaMemcpyAsync(sc + kOffJobs, jobs, njobs * sizeof(Job), cudaMemcpyHostToDevice, st) != cudaSuccess) return -1;
-    if (cudaMemcpyAsync(sc + kOffGrid, &G, sizeof(G), cudaMemcpyHostToDevice, st) != cudaSuccess) return -1;
-    if (tiles == 0) return 0;
-    build_worklist<<<1, 1024, 0, st>>>((const Job *)(sc + kOffJobs), njobs, (unsigned *)(sc + kOffCount),
-                                       (unsigned *)(sc + kOffCount) + kMaxDiag, items, maxd + 1);
+    MarchSet set;
+    set.n = 0;
+    for (int o = 0; o < 8; o++)
+        for (int a = 0; a < 3; a++)
+            if (make_march(set.m[set.n], nx, ny, nz, vtx, o, a, nx, false)) set.n++;
+    const int narr = n_dev ? 2 : 1;
+    const int rows = MarchShape<Real>::ROWS;
+    long long nitems = 0, cells = 0;
+    int itemdiag = 0;
+    for (int j = 0; j < set.n; j++) {
+        const int n1 = march_nt1(set.m[j]), n2 = march_nt2(set.m[j], rows);
+        nitems += (long long)n1 * n2;
+        itemdiag = std::max(itemdiag, n1 + n2 - 1);
+        for (int t = 0; t < n1 * n2; t++) {
+            MarchItem I;
+            cells += make_march_item(I, set.m[j], j, t % n1, t / n1, rows);
+        }
+    }
+    // the per-item arrays after the fixed part: progress words first (they must
+    // keep the tags of earlier launches, so their place does not move)
+    size_t off = items_offset<double>();
+    unsigned *progress = (unsigned *)(sc + off);
+    off += kMaxItems * sizeof(unsigned);
+    MarchItem *items = (MarchItem *)(sc + off);
+    off += kMaxItems * sizeof(MarchItem);
+    int *at = (int *)(sc + off);
+    off += kMaxItems * sizeof(int);
+    MCell<Real> *halo = (MCell<Real> *)(sc + off);
+    if (nitems > kMaxItems || itemdiag > kMaxItemDiag || off + (size_t)cells * sizeof(MCell<Real>) > kScratchBytes)
+        return -1000 - (int)std::min<long long>(tiles, 1 << 30);
+    if (nitems == 0) return 0;
+    build_worklist<Real><<<1, 1024, 0, st>>>(set, G, sc, rows, items, at, itemdiag);
     if (cudaGetLastError() != cudaSuccess) return -1;
 
-    SweepParams<Real> P;
+    MarchParams<Real> P;
     P.grids = (const GridDev<Real> *)(sc + kOffGrid);
-    P.jobs = (const Job *)(sc + kOffJobs);
+    P.marches = (const March *)(sc + kOffMarch);
     P.items = items;
-    P.nitems = (int)tiles;
+    P.nitems = (int)nitems;
     P.which = 0;
     P.ticket = (unsigned *)(sc + kOffTicket);
     P.done = (unsigned *)(sc + kOffTicket) + 1;
     P.epoch = (unsigned *)(sc + kOffEpoch);
-    P.faces = faces;
-    P.tpfaces = nullptr;
-    P.tpflags = nullptr;
-    P.tabs = nullptr;
+    P.halo = halo;
+    P.progress = progress;
     P.err = (int *)(sc + kOffErr);
     P.spin_limit = 1ll << 22;
     P.skip_publish = -1;
-    P.chunk = 0;
     P.ngrid = 0;
-    P.bricks = nullptr;
+    P.narr = narr;
     const int prec = sizeof(Real) == 8 ? 0 : 1;
-    if (launch_sweep<Real>(P, kShape, 0, S.nblocks[prec], st) != cudaSuccess) return -1;
+    if (launch_march<Real>(P, S.nblocks[prec][narr - 1], st) != cudaSuccess) return -1;
     return 0;
 }
 
@@ -230,19 +254,22 @@ extern "C" int oots_trace_noalloc(int device, int precision, int nx, int ny, int
     std::unique_lock<std::mutex> setup_lock(g_setup_mutex);
     if (!S.ready) {
         // once per device, with the device current: the device address of the
-        // static scratch (its host-side name is only a stand-in), the kernels'
-        // shared-memory opt-in, and the persistent grid size
+        // static scratch (its host-side name is only a stand-in) and the
+        // persistent grid sizes
         void *p = nullptr;
         if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) rc = OOTS_E_CUDA;
-        if (rc == OOTS_OK && (prepare_sweeps<double>() != cudaSuccess || prepare_sweeps<float>() != cudaSuccess))
-            rc = OOTS_E_CUDA;
         if (rc == OOTS_OK) {
             int nsm = 0;
             cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
             S.scratch = (unsigned char *)p;
-            S.nblocks[0] = sweep_occupancy<double>(kShape, 0) * nsm;
-            S.nblocks[1] = sweep_occupancy<float>(kShape, 0) * nsm;
-            S.ready = true;
+            for (int a = 0; a < 2 && rc == OOTS_OK; a++) {
+                int o64 = 0, o32 = 0;
+                if (march_occupancy<double>(a + 1, &o64) != cudaSuccess || march_occupancy<float>(a + 1, &o32) != cudaSuccess)
+                    rc = OOTS_E_CUDA;
+                S.nblocks[0][a] = o64 * nsm;
+                S.nblocks[1][a] = o32 * nsm;
+            }
+            S.ready = rc == OOTS_OK;
         }
     }
     setup_lock.unlock();

@@ -151,12 +151,17 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
     TileItem *d_items = nullptr;
     int nitems = 0;
     long long ntiles = 0;
-    unsigned *d_sync = nullptr;        // [0] ticket, [1] done (zeroed per sweep), [16] epoch (persistent)
+    unsigned *d_sync = nullptr;        // implicit sweep: [0] ticket, [1] done (zeroed per sweep), [16] epoch; march: [32], [33], [48]
     unsigned long long *d_faces = nullptr;
-    Real *d_tpfaces = nullptr;         // throughput sweep: untagged faces, and a flag per tile
-    unsigned *d_tpflags = nullptr;
-    Real *d_bricks = nullptr;          // throughput sweep: n x of every grid in bricks of the tile
-    long long brick_max = 0;           // brick cells of the largest grid (0: no bricks)
+    March *d_marches = nullptr;        // column march: pyramids, items, published halos, progress per item
+    MarchItem *d_mitems = nullptr;
+    int nmitems = 0;
+    int mblocks = 1;
+    int narr = 1;                      // its input arrays: 2 when some grid brings n and x unpacked
+    MCell<Real> *d_halo = nullptr;
+    unsigned *d_progress = nullptr;
+    Real *d_nxp = nullptr;             // n x of the traced state, packed (grids with many sources)
+    long long pack_max = 0;            // padded cells of the largest packed grid (0: none)
     PlaneJob *d_pjobs = nullptr;       // plane-parallel sources
     int npjobs = 0, nrow0 = 0;         // jobs; of them, rows along x (first in the array)
     long long plane_threads = 0, threads0 = 0;
@@ -171,7 +176,7 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
     unsigned *d_qcount = nullptr;      // queue lengths of the half and full integrations
     int gen_blocks = 1;                // grid of the general pass
     int cell_bs = 128;                 // threads per block of the closed-form passes
-    int nblocks0 = 1, nblocks1 = 1;
+    int nblocks1 = 1;
     int nsmax = 1;                     // largest source count among the grids
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
@@ -189,12 +194,14 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
         cudaFree(d_items);
         cudaFree(d_sync);
         cudaFree(d_faces);
-        cudaFree(d_tpfaces);
-        cudaFree(d_tpflags);
+        cudaFree(d_marches);
+        cudaFree(d_mitems);
+        cudaFree(d_halo);
+        cudaFree(d_progress);
+        cudaFree(d_nxp);
         cudaFree(d_pjobs);
         cudaFree(d_tabs);
         for (void *p : tabmem) cudaFree(p);
-        cudaFree(d_bricks);
         cudaFree(d_offsets);
         cudaFree(d_queue);
         cudaFree(d_qrec);
@@ -255,21 +262,22 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
         std::vector<DevTable<Real>> tabs;
         std::vector<long long> offs(cs.size());
         long long tile_base = 0, off = 0;
-        // the throughput kernel's traces read n x packed in bricks of the tile
-        // (tiles at global multiples of the tile only), one allocation for all grids
-        const bool pack = is_tp_shape(shape) && scheme != OOTS_A1;
-        std::vector<long long> brick_base(cs.size(), -1);
-        long long nbricks = 0;
+        std::vector<March> marches;
+        std::vector<long long> pack_base(cs.size(), -1);
+        long long packed = 0;
         for (size_t g = 0; g < cs.size(); g++) {
             oots_ctx *c = cs[g];
             GridDev<Real> &G = grids[g];
             memset(&G, 0, sizeof(G));
-            if (pack && !c->tile_align) {
-                G.nbx = (c->nx + TX - 1) / TX;
-                G.nby = (c->ny + TY - 1) / TY;
-                G.nbz = (c->nz + TZ - 1) / TZ;
-                brick_base[g] = nbricks;
-                nbricks += (long long)G.nbx * G.nby * G.nbz;
+            // With S sources the march reads n and x (8 B per cell) S times, or n x packed
+            // (4 B) S times after one pass that reads 8 B and writes 4 B: packing pays from S = 4.
+            G.pitch = c->nx;
+            if ((int)c->src.size() >= 4 && scheme != OOTS_A1) {
+                G.pitch = (c->nx + 7) / 8 * 8;
+                pack_base[g] = packed;
+                const long long pc = (long long)G.pitch * c->ny * c->nz;
+                packed += pc;
+                pack_max = std::max(pack_max, pc);
             }
             G.nx = c->nx; G.ny = c->ny; G.nz = c->nz;
             G.ncell = c->ncell;
@@ -321,6 +329,17 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
                     pjobs.push_back(P);
                     continue;
                 }
+                // (A1 traces only for a criterion on dx/dt)
+                for (int o = 0; o < 8 && (scheme != OOTS_A1 || c->crit.K3 > 0 || c->crit.K4 > 0); o++)
+                    for (int a = 0; a < 3; a++) {
+                        March M;
+                        if (!make_march(M, c->nx, c->ny, c->nz, S.v, o, a, G.pitch, pack_base[g] >= 0)) continue;
+                        if (pack_base[g] < 0 && G.n) narr = 2;
+                        M.grid = (int)g;
+                        M.src = s;
+                        marches.push_back(M);
+                    }
+                if (scheme != OOTS_A1) continue;
                 for (int o = 0; o < 8; o++) {
                     Job J;
                     memset(&J, 0, sizeof(J));
@@ -347,19 +366,7 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
                                 t.I = (unsigned short)I;
                                 t.J = (unsigned short)Jj;
                                 t.K = (unsigned short)K;
-                                t.grid = (unsigned short)g;
-                                t.brick = 0u;
-                                if (brick_base[g] >= 0) {
-                                    // lowest global cell of the tile along each axis (a multiple of the tile)
-                                    const int idx3[3] = {I, Jj, K};
-                                    long long b3[3];
-                                    for (int a = 0; a < 3; a++) {
-                                        const int o0 = idx3[a] * T3[a] - J.off[a];
-                                        const int lo = J.sg[a] > 0 ? J.v[a] + o0 : J.v[a] - o0 - T3[a];
-                                        b3[a] = lo / T3[a];
-                                    }
-                                    t.brick = (unsigned)(brick_base[g] + (b3[2] * G.nby + b3[1]) * G.nbx + b3[0]);
-                                }
+                                t.pad = 0;
                                 items.push_back(t);
                             }
                     tile_base += (long long)J.nt[0] * J.nt[1] * J.nt[2];
@@ -377,18 +384,10 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
         });
 
         CU(cudaSetDevice(device));
-        if (nbricks > 0 && !jobs.empty()) {
-            if (nbricks > 0xffffffffll) return fail(OOTS_E_INVAL, "%lld bricks in one call (32-bit brick indices)", nbricks);
-            const long long bc = (long long)TX * TY * TZ;
-            CU(cudaMalloc(&d_bricks, (size_t)(nbricks * bc) * sizeof(Real)));
-            for (size_t g = 0; g < cs.size(); g++) {
-                if (brick_base[g] < 0) continue;
-                GridDev<Real> &G = grids[g];
-                G.nxb = d_bricks + brick_base[g] * bc;
-                brick_max = std::max(brick_max, (long long)G.nbx * G.nby * G.nbz * bc);
-            }
-        } else {
-            for (auto &G : grids) G.nbx = G.nby = G.nbz = 0;
+        if (packed > 0) {
+            CU(cudaMalloc(&d_nxp, (size_t)packed * sizeof(Real)));
+            for (size_t g = 0; g < cs.size(); g++)
+                if (pack_base[g] >= 0) grids[g].nxp = d_nxp + pack_base[g];
         }
         if (nsmax > 1) {
             // each source's selection record, four copies per grid (dt pass, half step, full
@@ -433,27 +432,23 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
         CU(cudaMalloc(&d_rcache, (size_t)std::max(total, 1ll) * 3 * sizeof(Real)));
         CU(cudaMalloc(&d_qcount, 8 * sizeof(unsigned)));
         CU(cudaMemset(d_qcount, 0, 8 * sizeof(unsigned)));
+        if (!marches.empty() || !jobs.empty()) {
+            CU(cudaMalloc(&d_sync, 256));
+            CU(cudaMemset(d_sync, 0, 256));
+        }
+        if (!marches.empty()) {
+            int rc = build_march(marches, c0->nsm);
+            if (rc) return rc;
+        }
         if (!jobs.empty()) {
             CU(cudaMalloc(&d_jobs, jobs.size() * sizeof(Job)));
             CU(cudaMemcpy(d_jobs, jobs.data(), jobs.size() * sizeof(Job), cudaMemcpyHostToDevice));
             CU(cudaMalloc(&d_items, items.size() * sizeof(TileItem)));
             CU(cudaMemcpy(d_items, items.data(), items.size() * sizeof(TileItem), cudaMemcpyHostToDevice));
-            CU(cudaMalloc(&d_sync, 128));
-            CU(cudaMemset(d_sync, 0, 128));
-            // faces start with epoch 0 in every word (flags at 0); launches use epochs 1, 2, ...
-            // The pipelined kernel publishes tagged words; the throughput kernel
-            // (shape 7) plain values and a flag per tile; A1 runs the pipelined
-            // kernel on shape 7's tiles.
-            if (!is_tp_shape(shape) || scheme == OOTS_A1) {
-                const size_t fbytes = (size_t)ntiles * 3 * FMAX * face_words<Real>() * sizeof(unsigned long long);
-                CU(cudaMalloc(&d_faces, fbytes));
-                CU(cudaMemset(d_faces, 0, fbytes));
-            }
-            if (is_tp_shape(shape)) {
-                CU(cudaMalloc(&d_tpfaces, (size_t)ntiles * 3 * FMAX * tp_face_comps<Real>() * sizeof(Real)));
-                CU(cudaMalloc(&d_tpflags, (size_t)ntiles * sizeof(unsigned)));
-                CU(cudaMemset(d_tpflags, 0, (size_t)ntiles * sizeof(unsigned)));
-            }
+            // faces start with epoch 0 in every word; launches use epochs 1, 2, ...
+            const size_t fbytes = (size_t)ntiles * 3 * FMAX * face_words<Real>() * sizeof(unsigned long long);
+            CU(cudaMalloc(&d_faces, fbytes));
+            CU(cudaMemset(d_faces, 0, fbytes));
         }
         if (!pjobs.empty()) {
             // rows along x first (their trace kernel differs), then the rest
@@ -473,10 +468,9 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
             CU(cudaMalloc(&d_tabs, tabs.size() * sizeof(DevTable<Real>)));
             CU(cudaMemcpy(d_tabs, tabs.data(), tabs.size() * sizeof(DevTable<Real>), cudaMemcpyHostToDevice));
         }
-        CU(prepare_sweeps<Real>());
+        if (scheme == OOTS_A1) CU(prepare_sweeps<Real>());
         int nsm = c0->nsm;
-        nblocks0 = sweep_occupancy<Real>(shape, 0) * nsm;
-        nblocks1 = sweep_occupancy<Real>(shape, 1) * nsm;
+        if (scheme == OOTS_A1) nblocks1 = sweep_occupancy<Real>(shape) * nsm;
         gen_blocks = cell_general_occupancy<Real>(nsmax) * nsm;
         // closed-form passes: 128-thread blocks for many sources (a slow cell holds up fewer others),
         // 256 for one source (cheap cells; fewer block set-ups), unless tuned
@@ -484,27 +478,98 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
         return OOTS_OK;
     }
 
-    SweepParams<Real> params(int which) const
+    // The march's work list: the blocks of every pyramid, handed out in order of
+    // T1 + T2 (an item's upstream blocks come first), longer ones first among equals.
+    int build_march(const std::vector<March> &marches, int nsm)
+    {
+        const int rows = MarchShape<Real>::ROWS;
+        std::vector<MarchItem> list;
+        std::vector<long long> first(marches.size()), pubs;
+        for (size_t m = 0; m < marches.size(); m++) {
+            const int n1 = march_nt1(marches[m]), n2 = march_nt2(marches[m], rows);
+            first[m] = (long long)list.size();
+            for (int T2 = 0; T2 < n2; T2++)
+                for (int T1 = 0; T1 < n1; T1++) {
+                    MarchItem I;
+                    pubs.push_back(make_march_item(I, marches[m], (int)m, T1, T2, rows));
+                    list.push_back(I);
+                }
+        }
+        if (list.size() > 0x7fffffffull) return fail(OOTS_E_INVAL, "%zu blocks in one trace", list.size());
+        std::vector<int> order(list.size()), at(list.size());
+        for (size_t i = 0; i < list.size(); i++) order[i] = (int)i;
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+            const MarchItem &A = list[a], &B = list[b];
+            const int da = A.T1 + A.T2, db = B.T1 + B.T2;
+            if (da != db) return da < db;
+            return marches[A.march].len - A.l0 > marches[B.march].len - B.l0;
+        });
+        for (size_t i = 0; i < order.size(); i++) at[order[i]] = (int)i;
+        std::vector<MarchItem> items(list.size());
+        long long cells = 0;
+        for (size_t i = 0; i < order.size(); i++) {
+            MarchItem I = list[order[i]];
+            const int n1 = march_nt1(marches[I.march]);
+            const long long lin = first[I.march] + (long long)I.T2 * n1 + I.T1;
+            if (I.T1 > 0) I.up0 = at[lin - 1];
+            if (I.T2 > 0) I.up1 = at[lin - n1];
+            if (I.T1 > 0 && I.T2 > 0) I.up2 = at[lin - n1 - 1];
+            I.halo = cells;
+            cells += pubs[order[i]];
+            items[i] = I;
+        }
+        nmitems = (int)items.size();
+        CU(cudaMalloc(&d_marches, marches.size() * sizeof(March)));
+        CU(cudaMemcpy(d_marches, marches.data(), marches.size() * sizeof(March), cudaMemcpyHostToDevice));
+        CU(cudaMalloc(&d_mitems, items.size() * sizeof(MarchItem)));
+        CU(cudaMemcpy(d_mitems, items.data(), items.size() * sizeof(MarchItem), cudaMemcpyHostToDevice));
+        CU(cudaMalloc(&d_halo, (size_t)std::max(cells, 1ll) * sizeof(MCell<Real>)));
+        CU(cudaMalloc(&d_progress, items.size() * sizeof(unsigned)));
+        CU(cudaMemset(d_progress, 0, items.size() * sizeof(unsigned)));
+        int per_sm = 0;
+        CU(march_occupancy<Real>(narr, &per_sm));
+        mblocks = per_sm * nsm;
+        return OOTS_OK;
+    }
+
+    MarchParams<Real> march_params(int which) const
+    {
+        MarchParams<Real> P;
+        P.grids = d_grids;
+        P.marches = d_marches;
+        P.items = d_mitems;
+        P.nitems = nmitems;
+        P.which = which;
+        P.ticket = d_sync + 32;
+        P.done = d_sync + 33;
+        P.epoch = d_sync + 48;
+        P.halo = d_halo;
+        P.progress = d_progress;
+        P.err = d_err;
+        P.spin_limit = spin_limit;
+        P.skip_publish = skip_publish;
+        P.ngrid = (int)ctxs.size();
+        P.narr = narr;
+        return P;
+    }
+
+    SweepParams<Real> params() const
     {
         SweepParams<Real> P;
         P.grids = d_grids;
         P.jobs = d_jobs;
         P.items = d_items;
         P.nitems = nitems;
-        P.which = which;
         P.ticket = d_sync;
         P.done = d_sync + 1;
         P.epoch = d_sync + 16;
         P.faces = d_faces;
-        P.tpfaces = d_tpfaces;
-        P.tpflags = d_tpflags;
         P.tabs = d_tabs;
         P.err = d_err;
         P.spin_limit = spin_limit;
         P.skip_publish = skip_publish;
         P.chunk = sweep_chunk;
         P.ngrid = (int)ctxs.size();
-        P.bricks = d_bricks;
         return P;
     }
 
@@ -512,17 +577,22 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
     // sources by the wavefront sweep, plane sources row by row
     int sweep(cudaStream_t s, int which, int mode)
     {
-        if (nitems > 0) {
-            CU(cudaMemsetAsync(d_sync, 0, 2 * sizeof(unsigned), s));   // ticket and done; the epoch persists
+        if (mode == 0 && nmitems > 0) {
             if (prof) prof->mark(0);
-            // the trace's input in bricks (timed with the trace)
-            if (mode == 0 && brick_max > 0) {
-                CU(launch_pack_nx<Real>(d_grids, (int)ctxs.size(), which, shape, brick_max, ctxs[0]->nsm, s));
+            if (pack_max > 0) {
+                // the trace's input packed
+                CU(launch_pack_nx<Real>(d_grids, (int)ctxs.size(), which, pack_max, ctxs[0]->nsm, s));
                 if (prof) prof->mark(OOTS_K_PACK);
                 if (prof) prof->mark(0);
             }
-            CU(launch_sweep<Real>(params(which), shape, mode, mode == 0 ? nblocks0 : nblocks1, s));
-            if (prof) prof->mark(mode == 1 ? OOTS_K_IMPLICIT : (which == 0 ? OOTS_K_SWEEP1 : OOTS_K_SWEEP2));
+            CU(launch_march<Real>(march_params(which), mblocks, s));
+            if (prof) prof->mark(which == 0 ? OOTS_K_SWEEP1 : OOTS_K_SWEEP2);
+        }
+        if (mode == 1 && nitems > 0) {
+            CU(cudaMemsetAsync(d_sync, 0, 2 * sizeof(unsigned), s));   // ticket and done; the epoch persists
+            if (prof) prof->mark(0);
+            CU(launch_sweep<Real>(params(), shape, nblocks1, s));
+            if (prof) prof->mark(OOTS_K_IMPLICIT);
         }
         if (npjobs > 0) {
             if (prof) prof->mark(0);

@@ -34,11 +34,36 @@ struct PlaneJob {
     long long first;       // first thread of the job in the launch (a multiple of 256)
 };
 
-// One tile of a job, ordered in the work list by tile diagonal I+J+K.  grid:
-// the job's grid (as Job::grid; launches of at most 65535 grids).  brick: the
-// tile's brick in the launch's packed n x (GridDev::nxb counts from the same
-// base), when the launch packs its input (throughput tiles).
-struct TileItem { int job; unsigned short I, J, K, grid; unsigned brick; };
+// One tile of a job, ordered in the work list by tile diagonal I+J+K.
+struct TileItem { int job; unsigned short I, J, K, pad; };
+
+// One pyramid of the column march (march.cuh): the cells of one octant of one
+// source whose dominant axis is `axis`, layer l of that axis holding the cells
+// u, w <= l of the other two.  u is x unless the axis is x (then y); w is the
+// remaining axis.  Indices of cell (l, u, w): base + l sl + u su + w sw, in the
+// input (rows of `pitch` values when packed) and in the grid's own layout; the
+// stride along x is the sign sg (so sl of axis 0 and su of the others are not
+// stored).
+struct March {
+    int grid, src, axis, sg;
+    int len, eu, ew;          // layers; cells along u and w
+    int off;                  // layers go in chunks of eight from layer -off (axis x: whole sectors of x)
+    int packed;               // the input is n x in padded rows (GridDev::nxp)
+    int pad[3];
+    long long ibase, isl, isu, isw;
+    long long obase, osl, osu, osw;
+};
+
+// One work item of the march: block (T1, T2) of a pyramid, layers l0 and up.
+struct MarchItem {
+    int march, l0;
+    unsigned short T1, T2;
+    unsigned char right, above;   // some item reads this one's right column / top row
+    unsigned short pad;
+    int up0, up1, up2;            // the items to the left, below and below left (-1: none)
+    int pad2;
+    long long halo;               // first published cell (MCell) of this item
+};
 
 // Per-grid state that lives on the device, read and written by the kernels
 // (so that substeps can be replayed from a CUDA graph without host sync).
@@ -96,10 +121,8 @@ template <typename Real> struct GridDev {
     int tab[MAX_SRC];         // -1 monochromatic, else table index
     unsigned char pcode[MAX_SRC];  // 0: vertex point source; 1 + 2*axis + back: plane source (qfac = F/dx)
     float lnamp0[MAX_SRC];    // ln(qfac sigma0 dx): a source's largest rate per unit x is qfac sigma0 dx p / r2
-    Real *nxb;                // n x of the traced state in bricks of the throughput tile (nullptr: none):
-                              // brick (bx, by, bz) of nbx x nby x nbz holds cells bx*TX.., by*8.., bz*8..,
-                              // x fastest, TX = the tile's x extent
-    int nbx, nby, nbz;
+    Real *nxp;                // n x of the traced state in rows of `pitch` values (nullptr: none)
+    int pitch;
     SrcSel<Real> *sel;        // 4 x MAX_SRC source records for the dt pass (nst: the column beyond which
                               // a source cannot matter within the step hint), the half step, the full
                               // step and the verifying dt pass (nst = +inf); nullptr: one source

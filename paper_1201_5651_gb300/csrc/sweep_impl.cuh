@@ -277,12 +277,13 @@ template <typename Real> __device__ __forceinline__ bool sweep_live(const SweepP
     return false;
 }
 
-template <typename Real, int TX, int TY, int TZ, int MODE>
+template <typename Real, int TX, int TY, int TZ>
 __global__ void __launch_bounds__(TY *TZ + 64)
 sweep_kernel(SweepParams<Real> P)
 {
     typedef typename ColT<Real>::type Col;
     typedef TileLayout<TX, TY, TZ> L;
+    constexpr int MODE = 1;
     constexpr int NT = L::NT;                    // chain threads
     constexpr int NC = TX * TY * TZ;
     constexpr int NP = L::NP;
@@ -368,7 +369,7 @@ sweep_kernel(SweepParams<Real> P)
         const GridDev<Real> &G = P.grids[J.grid];
         const int i0 = it.I * TX - J.off[0], j0 = it.J * TY - J.off[1], k0 = it.K * TZ - J.off[2];
         const long long tile_self = J.tile_base + ((long long)it.K * J.nt[1] + it.J) * J.nt[0] + it.I;
-        const Real *xin = (P.which == 1) ? G.xh : G.x;
+        const Real *xin = G.x;
         const Real dx = G.dx, sig = G.sigma0, tau0 = G.tau0;
 
         if (tid >= NT + 32) {
@@ -720,7 +721,7 @@ sweep_kernel(SweepParams<Real> P)
             }
 
             // 4. entry columns of the tile's cells
-            Real *Nout = (P.which == 1 ? G.N2 : G.N1) + (long long)J.src * G.ncell;
+            Real *Nout = G.N1 + (long long)J.src * G.ncell;
             for (int e = tid; e < NC; e += NT) {
                 const int li = e % TX, lj = (e / TX) % TY, lk = e / (TX * TY);
                 const int i = i0 + li, j = j0 + lj, k = k0 + lk;
@@ -756,12 +757,6 @@ sweep_kernel(SweepParams<Real> P)
     if (tid == 0 && atomicAdd(P.done, 1u) == gridDim.x - 1) *(volatile unsigned *)P.epoch = epoch;
 }
 
-} // namespace oots
-
-#include "sweep_tp.cuh"
-
-namespace oots {
-
 // ---------------------------------------------------------------------------
 // Launch wrappers
 // ---------------------------------------------------------------------------
@@ -769,14 +764,6 @@ template <typename Real, int TX, int TY, int TZ>
 constexpr size_t sweep_smem()
 {
     return (size_t)TileLayout<TX, TY, TZ>::HSZ * (sizeof(typename ColT<Real>::type) + 5 * sizeof(Real) + 1);
-}
-
-template <typename Real, int TX, int TY, int TZ, int MODE>
-static cudaError_t launch_shape(const SweepParams<Real> &P, int nblocks, cudaStream_t s)
-{
-    constexpr size_t sm = sweep_smem<Real, TX, TY, TZ>();
-    sweep_kernel<Real, TX, TY, TZ, MODE><<<nblocks, TY * TZ + 64, sm, s>>>(P);
-    return cudaGetLastError();
 }
 
 // Largest dynamic shared memory a block may use on this device.
@@ -788,19 +775,10 @@ static int max_optin_smem()
     return v;
 }
 
-template <typename Real, int TX, int TY, int TZ, int MODE>
-static cudaError_t prepare_shape()
-{
-    constexpr size_t sm = sweep_smem<Real, TX, TY, TZ>();
-    if ((int)sm > max_optin_smem()) return cudaSuccess;     // shape unavailable at this precision
-    return cudaFuncSetAttribute(sweep_kernel<Real, TX, TY, TZ, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-}
-
 template <typename Real>
 bool sweep_shape_ok(int shape)
 {
-    if (shape == SHAPE_TP8) return (int)sweep_tp_smem<Real, 8>() <= max_optin_smem() && sweep_shape_ok<Real>(4);
-    if (shape == SHAPE_TP16) return (int)sweep_tp_smem<Real, 16>() <= max_optin_smem() && sweep_shape_ok<Real>(0);
+    shape = sweep_twin(shape);
     size_t sm = 0;
 #define OOTS_SM(ID, TX, TY, TZ) if (shape == ID) sm = sweep_smem<Real, TX, TY, TZ>();
     OOTS_SHAPES(OOTS_SM)
@@ -809,23 +787,15 @@ bool sweep_shape_ok(int shape)
 }
 
 template <typename Real>
-int sweep_occupancy(int shape, int mode)
+int sweep_occupancy(int shape)
 {
     int nb = 0;
     cudaError_t e = cudaSuccess;
-    if (is_tp_shape(shape)) {
-        if (mode == 1) return sweep_occupancy<Real>(tp_twin(shape), 1);
-        if (shape == SHAPE_TP8)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_tp_kernel<Real, 8>, 64, sweep_tp_smem<Real, 8>());
-        else
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_tp_kernel<Real, 16>, 64, sweep_tp_smem<Real, 16>());
-        return (e == cudaSuccess && nb > 0) ? nb : 1;
-    }
+    shape = sweep_twin(shape);
 #define OOTS_OCC(ID, TX, TY, TZ)                                                                      \
     if (shape == ID) {                                                                                \
         constexpr size_t sm = sweep_smem<Real, TX, TY, TZ>();                                         \
-        if (mode == 0) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<Real, TX, TY, TZ, 0>, TY * TZ + 64, sm); \
-        else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<Real, TX, TY, TZ, 1>, TY * TZ + 64, sm); \
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<Real, TX, TY, TZ>, TY * TZ + 64, sm); \
     }
     OOTS_SHAPES(OOTS_OCC)
 #undef OOTS_OCC
@@ -834,22 +804,17 @@ int sweep_occupancy(int shape, int mode)
 }
 
 template <typename Real>
-cudaError_t launch_sweep(const SweepParams<Real> &P, int shape, int mode, int nblocks, cudaStream_t s)
+cudaError_t launch_sweep(const SweepParams<Real> &P, int shape, int nblocks, cudaStream_t s)
 {
     if (P.nitems <= 0) return cudaSuccess;
     long long nb = nblocks;
     if (nb > P.nitems) nb = P.nitems;
     if (nb < 1) nb = 1;
-    if (is_tp_shape(shape)) {
-        if (mode == 1) return launch_sweep<Real>(P, tp_twin(shape), 1, nblocks, s);
-        if (shape == SHAPE_TP8) sweep_tp_kernel<Real, 8><<<(int)nb, 64, sweep_tp_smem<Real, 8>(), s>>>(P);
-        else sweep_tp_kernel<Real, 16><<<(int)nb, 64, sweep_tp_smem<Real, 16>(), s>>>(P);
-        return cudaGetLastError();
-    }
-#define OOTS_LAUNCH(ID, TX, TY, TZ)                                                         \
-    if (shape == ID) {                                                                      \
-        return mode == 0 ? launch_shape<Real, TX, TY, TZ, 0>(P, (int)nb, s)                 \
-                         : launch_shape<Real, TX, TY, TZ, 1>(P, (int)nb, s);                \
+    shape = sweep_twin(shape);
+#define OOTS_LAUNCH(ID, TX, TY, TZ)                                                                          \
+    if (shape == ID) {                                                                                       \
+        sweep_kernel<Real, TX, TY, TZ><<<(int)nb, TY * TZ + 64, sweep_smem<Real, TX, TY, TZ>(), s>>>(P);     \
+        return cudaGetLastError();                                                                           \
     }
     OOTS_SHAPES(OOTS_LAUNCH)
 #undef OOTS_LAUNCH
@@ -857,41 +822,18 @@ cudaError_t launch_sweep(const SweepParams<Real> &P, int shape, int mode, int nb
 }
 
 template <typename Real>
-cudaError_t launch_pack_nx(const GridDev<Real> *grids, int ngrid, int which, int shape, long long max_elems, int nsm,
-                           cudaStream_t s)
-{
-    if (ngrid <= 0 || max_elems <= 0) return cudaSuccess;
-    if (ngrid > 65535) return cudaErrorInvalidValue;
-    long long nb = (max_elems + 255) / 256;
-    const long long cap = (long long)(nsm > 0 ? nsm : 1) * 8;       // 2048 threads per SM
-    if (nb > cap) nb = cap;
-    const dim3 grid((unsigned)nb, (unsigned)ngrid);
-    if (shape == SHAPE_TP16) pack_nx_kernel<Real, 16><<<grid, 256, 0, s>>>(grids, which);
-    else pack_nx_kernel<Real, 8><<<grid, 256, 0, s>>>(grids, which);
-    return cudaGetLastError();
-}
-
-template <typename Real>
 cudaError_t prepare_sweeps()
 {
     cudaError_t e = cudaSuccess, e2;
-#define OOTS_PREP(ID, TX, TY, TZ)                                  \
-    e2 = prepare_shape<Real, TX, TY, TZ, 0>(); if (e2 != cudaSuccess) e = e2; \
-    e2 = prepare_shape<Real, TX, TY, TZ, 1>(); if (e2 != cudaSuccess) e = e2;
+#define OOTS_PREP(ID, TX, TY, TZ)                                                                            \
+    if ((int)sweep_smem<Real, TX, TY, TZ>() <= max_optin_smem()) {                                           \
+        e2 = cudaFuncSetAttribute(sweep_kernel<Real, TX, TY, TZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                  (int)sweep_smem<Real, TX, TY, TZ>());                                      \
+        if (e2 != cudaSuccess) e = e2;                                                                       \
+    }
     OOTS_SHAPES(OOTS_PREP)
 #undef OOTS_PREP
-    if ((int)sweep_tp_smem<Real, 8>() <= max_optin_smem()) {
-        e2 = cudaFuncSetAttribute(sweep_tp_kernel<Real, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)sweep_tp_smem<Real, 8>());
-        if (e2 != cudaSuccess) e = e2;
-    }
-    if ((int)sweep_tp_smem<Real, 16>() <= max_optin_smem()) {
-        e2 = cudaFuncSetAttribute(sweep_tp_kernel<Real, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)sweep_tp_smem<Real, 16>());
-        if (e2 != cudaSuccess) e = e2;
-    }
     return e;
 }
-
 
 } // namespace oots
