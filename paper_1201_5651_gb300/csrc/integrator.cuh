@@ -74,20 +74,25 @@ OOTS_HD __forceinline__ void leg_coeffs(const Real *v, Real *c)
     for (int n = 0; n < G; n++) c[n] *= Real(2 * n + 1) * Real(0.5);
 }
 
-// int_s^1 of the interpolant (Legendre coefficients c) and its value at s.
-// The interpolant has degree G-1, so the G-point Gauss rule on [s, 1] gives its
-// integral exactly, with no cancellation as s -> 1.
+// Sum of c_n P_n(t) by Clenshaw's recurrence (its factors are compile-time
+// constants: no division; forming P_0 .. P_{G-1} divided by n + 1 at every
+// step, which made the inversions below the larger part of a cell's work).
 template <typename Real, int G>
 OOTS_HD __forceinline__ Real leg_eval(const Real *c, Real t)
 {
-    Real P[G];
-    legendre<Real, G>(t, P);
-    Real v = Real(0);
+    Real b1 = c[G - 1], b2 = Real(0);
 #pragma unroll
-    for (int n = 0; n < G; n++) v += c[n] * P[n];
-    return v;
+    for (int k = G - 2; k >= 1; k--) {
+        const Real b0 = c[k] + (Real(2 * k + 1) / Real(k + 1)) * t * b1 - (Real(k + 1) / Real(k + 2)) * b2;
+        b2 = b1;
+        b1 = b0;
+    }
+    return c[0] + t * b1 - Real(0.5) * b2;
 }
 
+// int_s^1 of the interpolant (Legendre coefficients c) and its value at s.
+// The interpolant has degree G-1, so the G-point Gauss rule on [s, 1] gives its
+// integral exactly, with no cancellation as s -> 1.
 template <typename Real, int G>
 OOTS_HD __forceinline__ void leg_tail(const Real *c, Real s, Real *integral, Real *value)
 {
@@ -192,12 +197,25 @@ template <> struct IntCfg<double> {
     static OOTS_HD double umax() { return 40.0; }
     static OOTS_HD double tolq() { return 1e-14; }
     static OOTS_HD double zlin() { return 1e-6; }    // linearised step allowed below this h|f'|
+    // series step: terms, largest h|f'| (z^9/9! is 3e-15 there) and largest change in units of the bending
+    // scale 1/b (the cubic through both ends is then off by delta^4/384 = 7e-13 of f)
+    enum { KSER = 8 };
+    static OOTS_HD double zser() { return 0.08; }
+    static OOTS_HD double dser() { return 4e-3; }
+    // near the root: largest b |x0 - x_eq| when the step relaxes it by e^-45, and at all with A1's average
+    static OOTS_HD double drel() { return 4e-3; }
+    static OOTS_HD double davg() { return 1e-6; }
 };
 template <> struct IntCfg<float> {
     enum { G = 4 };
     static OOTS_HD float umax() { return 20.0f; }
     static OOTS_HD float tolq() { return 1e-6f; }
     static OOTS_HD float zlin() { return 3e-3f; }
+    enum { KSER = 5 };
+    static OOTS_HD float zser() { return 0.2f; }
+    static OOTS_HD float dser() { return 0.1f; }
+    static OOTS_HD float drel() { return 2e-2f; }
+    static OOTS_HD float davg() { return 3e-4f; }
 };
 
 template <typename Real, int NSMAX>
@@ -234,7 +252,7 @@ OOTS_HD Real newton_root(const CellODE<Real> &C, Real lo, Real hi, Real xk, Real
 }
 
 // Evaluators of the general path.
-//  - root(C, x0, f0, F0, dF0): the root x_eq of f.
+//  - root(C, x0, f0, F0, dF0, sigma0): the root x_eq of f.
 //  - eval<N>(node, invD, dv): fills invD[l] = 1/D and dv[l] = d at the N
 //    quadrature nodes l = 0..N-1, where node(l, d) returns 1/D at node l and
 //    sets its deviation d.
@@ -246,9 +264,22 @@ OOTS_HD Real newton_root(const CellODE<Real> &C, Real lo, Real hi, Real xk, Real
 struct SeqEval {
     static constexpr bool attenuation = true;    // A1's time-averaged attenuation when b0 > 0
     template <typename Real, int NSMAX>
-    OOTS_HD Real root(const CellODE<Real> &C, Real x0, Real f0, Real F0, Real dF0) const
+    OOTS_HD Real root(const CellODE<Real> &C, Real x0, Real f0, Real F0, Real dF0, Real sigma0) const
     {
         const Real lo = f0 > Real(0) ? x0 : Real(0), hi = f0 > Real(0) ? Real(1) : x0;
+        if (f0 < Real(0)) {
+            // from the right, Newton undershoots and then halves its way down whenever the rate
+            // saturates between the root and x0; from x = 0, left of the root, it rises to it
+            // without overshooting (f is convex)
+            Real bx = Real(0);
+            for (int i = 0; i < NSMAX && i < C.ns; i++)
+                if (C.r[i].A > Real(0)) bx = m_max(bx, C.r[i].tab < 0 ? C.r[i].b : sigma0 * C.r[i].b);
+            if (bx * x0 > Real(0.5)) {
+                Real F, dF;
+                ode_F<Real, NSMAX>(C, Real(0), &F, &dF);
+                return newton_root<Real, NSMAX>(C, lo, hi, Real(0), C.c, Real(0), -dF - Real(2) * C.c);
+            }
+        }
         return newton_root<Real, NSMAX>(C, lo, hi, x0, f0, F0, -dF0 - Real(2) * C.c * (Real(1) - x0));
     }
     template <int N, typename Real, typename Node>
@@ -275,7 +306,7 @@ template <int W> struct GroupEval {
     // of the root, so the ballot of f > 0 marks the lanes below it.  Newton
     // polishes from the left end of the sign change.
     template <typename Real, int NSMAX>
-    __device__ Real root(const CellODE<Real> &C, Real x0, Real f0, Real F0, Real dF0) const
+    __device__ Real root(const CellODE<Real> &C, Real x0, Real f0, Real F0, Real dF0, Real) const
     {
         const bool above = f0 > Real(0);                     // root in (x0, 1]
         const Real span = above ? Real(1) - x0 : x0;
@@ -346,22 +377,97 @@ OOTS_HD void root_slope(const CellODE<Real> &C, Real xe, Real sigma0, SrcEq<Real
 }
 
 // Already next to the root (|d0| = |x0 - x_eq| far below both bending scales):
-// the linearised solution about x_eq, d(t) = d0 e^{-Dinf t}.  Returns false
-// when the state is not that close.
+// the linearised solution about x_eq, d(t) = d0 e^{-Dinf t}.  A step that
+// relaxes the deviation by e^-45 leaves x = x_eq whatever its path, which only
+// the small time integrals see, so the deviation may be larger there.  Returns
+// false when the state is not that close.
 template <typename Real>
 OOTS_HD bool near_root_solution(const CellODE<Real> &C, Real xe, Real d0, Real Dinf, Real bmax, Real h,
                                 IntResult<Real> &R)
 {
-    const Real ad0 = m_abs(d0);
-    if (!(bmax * ad0 <= IntCfg<Real>::zlin() && ad0 <= IntCfg<Real>::zlin() * (Real(1) - xe) && C.b0 == Real(0)))
-        return false;
-    const Real e = m_exp(-Dinf * h);
+    const Real ad0 = m_abs(d0), one = Real(1) - xe, q = Dinf * h;
+    const Real lim = C.b0 > Real(0) ? IntCfg<Real>::davg() : (q > Real(45) ? IntCfg<Real>::drel() : IntCfg<Real>::zlin());
+    if (!(bmax * ad0 <= lim && ad0 <= lim * one)) return false;
+    const Real e = m_exp(-q);
     R.x = xe + d0 * e;
-    const Real one = Real(1) - xe;
     // int c (1 - xe - d)^2 dt = c one^2 h - 2 c one d0 (1 - e)/Dinf + c d0^2 (1 - e^2)/(2 Dinf)
-    const Real g1 = (Dinf * h > Real(1e-6)) ? -m_expm1(-Dinf * h) / Dinf : h;
-    const Real g2 = (Dinf * h > Real(1e-6)) ? -m_expm1(Real(-2) * Dinf * h) / (Real(2) * Dinf) : h;
+    const Real g1 = (q > Real(1e-6)) ? -m_expm1(-q) / Dinf : h;
+    const Real g2 = (q > Real(1e-6)) ? -m_expm1(Real(-2) * q) / (Real(2) * Dinf) : h;
     R.IR = C.c * (one * one * h - Real(2) * one * d0 * g1 + d0 * d0 * g2);
+    if (C.b0 > Real(0)) {
+        // mean of exp(-b0 (xe + d)), b0 d at most davg
+        const Real y = C.b0 * d0;
+        R.lnfav = -C.b0 * xe + m_log1p((Real(0.5) * y * y * g2 - y * g1) / h);
+    }
+    return true;
+}
+
+// Step of a slow cell: h |f'| and the change of x in units of every bending
+// scale are small.  f on the way is the cubic through its values and slopes at
+// x0 and at the linearised end of the step (exact for the recombination term),
+// and the solution of dx/dt = cubic is its power series in t, whose
+// coefficients follow from one another by Cauchy products.  One evaluation of
+// the rates; the quadrature spends 24 and more, and before this form took nine
+// in ten of the cells that the FP64 path queued.  bm: largest 1/scale; returns
+// false when the cell is not that slow.
+template <typename Real, int NSMAX>
+OOTS_HD bool series_step(const CellODE<Real> &C, Real x0, Real h, Real f0, Real df0, Real bm, IntResult<Real> &R)
+{
+    constexpr int K = IntCfg<Real>::KSER, G = IntCfg<Real>::G;
+    const Real z = h * df0;
+    if (!(m_abs(z) <= IntCfg<Real>::zser())) return false;
+    const Real phi = (m_abs(z) > Real(1e-8)) ? m_expm1(z) / z : Real(1) + Real(0.5) * z;
+    const Real D = h * f0 * phi, ad = m_abs(D), del = bm * ad, x1 = x0 + D;
+    if (!(del <= IntCfg<Real>::dser() && x1 >= Real(0) && x1 <= Real(1) && x1 >= Real(0.5) * x0 && ad > Real(0))) return false;
+    // what the cubic leaves out, against the rounding of x
+    if (!(ad * del * del * del * del <= Real(100) * RealLimits<Real>::eps() * x0)) return false;
+    Real F1, dF1;
+    ode_F<Real, NSMAX>(C, x1, &F1, &dF1);
+    const Real f1 = -F1 + C.c * (Real(1) - x1) * (Real(1) - x1);
+    const Real df1 = -dF1 - Real(2) * C.c * (Real(1) - x1);
+    // f(x0 + s) = f0 + a1 s + a2 s^2 + a3 s^3, in units of the step: s = D y, coefficients times h/D
+    const Real hd = h / D, a0 = hd * f0, a1 = z, b1 = h * df1, dd = hd * (f1 - f0);
+    const Real a2 = Real(3) * dd - Real(2) * a1 - b1, a3 = a1 + b1 - Real(2) * dd;
+    Real S[K + 1], Q[K + 1], T[K + 1];          // y, y^2, y^3 as power series in t/h
+    S[0] = Q[0] = T[0] = Real(0);
+    S[1] = a0;
+    Q[1] = T[1] = Real(0);
+#pragma unroll
+    for (int k = 1; k < K; k++) {
+        if (k > 1) {
+            Q[k] = T[k] = Real(0);
+#pragma unroll
+            for (int i = 1; i < k; i++) { Q[k] += S[i] * S[k - i]; T[k] += Q[i] * S[k - i]; }
+        }
+        S[k + 1] = (a1 * S[k] + a2 * Q[k] + a3 * T[k]) * (Real(1) / Real(k + 1));
+    }
+    Q[K] = Real(0);
+#pragma unroll
+    for (int i = 1; i < K; i++) Q[K] += S[i] * S[K - i];
+    Real y = Real(0), iy = Real(0), iq = Real(0);   // y at the end, mean of y and of y^2
+#pragma unroll
+    for (int k = K; k >= 1; k--) {
+        y += S[k];
+        iy += S[k] * (Real(1) / Real(k + 1));
+        iq += Q[k] * (Real(1) / Real(k + 1));
+    }
+    const Real xn = x0 + D * y, one = Real(1) - x0;
+    if (!(xn >= Real(0) && xn <= Real(1))) return false;
+    R.x = xn;
+    R.IR = C.c * h * (one * one - Real(2) * one * D * iy + D * D * iq);
+    if (C.b0 > Real(0)) {
+        // mean of exp(-b0 (x - x0)) over the step
+        Real acc = Real(0);
+#pragma unroll
+        for (int g = 0; g < G; g++) {
+            const Real t = Real(0.5) * (Real(1) + GL<G>::template x<Real>(g));
+            Real v = S[K];
+#pragma unroll
+            for (int k = K - 1; k >= 1; k--) v = v * t + S[k];
+            acc += GL<G>::template w<Real>(g) * Real(0.5) * m_expm1(-C.b0 * D * (v * t));
+        }
+        R.lnfav = -C.b0 * x0 + m_log1p(acc);
+    }
     return true;
 }
 
@@ -429,15 +535,15 @@ OOTS_HD bool integrate_prelude(const CellODE<Real> &C, Real x0, Real h, Real sig
     // the scales on which f bends (1/b of every source, and 1 - x for the
     // recombination term), the linearised solution x0 + f0 (e^{h f'} - 1)/f'
     // is exact to the working tolerance; IR by the midpoint rule
+    const Real df0 = -dF0 - Real(2) * C.c * (Real(1) - x0);
+    Real bm = C.b0;
+    for (int i = 0; i < NSMAX && i < C.ns; i++)
+        if (C.r[i].A > Real(0)) bm = m_max(bm, C.r[i].tab < 0 ? C.r[i].b : sigma0 * C.r[i].b);
     if (C.b0 == Real(0)) {
-        const Real df0 = -dF0 - Real(2) * C.c * (Real(1) - x0);
         const Real z = h * df0;
         if (m_abs(z) <= IntCfg<Real>::zlin()) {
             const Real phi = (m_abs(z) > Real(1e-8)) ? m_expm1(z) / z : Real(1) + Real(0.5) * z;
             const Real dx = h * f0 * phi;
-            Real bm = Real(0);
-            for (int i = 0; i < NSMAX && i < C.ns; i++)
-                if (C.r[i].A > Real(0)) bm = m_max(bm, C.r[i].tab < 0 ? C.r[i].b : sigma0 * C.r[i].b);
             const Real adx = m_abs(dx);
             // photoionisation bends on 1/b; the recombination term's curvature 2c
             // changes the increment by ~ c h dx relative
@@ -449,35 +555,32 @@ OOTS_HD bool integrate_prelude(const CellODE<Real> &C, Real x0, Real h, Real sig
                 return true;
             }
         }
-        // near the root: when one Newton step puts x_eq within both bending
-        // scales of x0, up to three Newton steps find it (f is smooth there)
-        // and the linearised solution about it finishes the cell
-        Real bm = Real(0);
-        for (int i = 0; i < NSMAX && i < C.ns; i++)
-            if (C.r[i].A > Real(0)) bm = m_max(bm, C.r[i].tab < 0 ? C.r[i].b : sigma0 * C.r[i].b);
-        const Real est = df0 < Real(0) ? m_abs(f0 / df0) : RealLimits<Real>::inf();
-        if (bm * est <= IntCfg<Real>::zlin() && est <= IntCfg<Real>::zlin() * (Real(1) - x0 + est)) {
-            Real xk = x0, fk = f0, Fk = F0, dfk = df0;
-            bool conv = false;
-            for (int it = 0; it < 3 && dfk < Real(0); it++) {
-                xk = m_min(m_max(xk - fk / dfk, Real(0)), Real(1));
-                Real dFk;
-                ode_F<Real, NSMAX>(C, xk, &Fk, &dFk);
-                fk = -Fk + C.c * (Real(1) - xk) * (Real(1) - xk);
-                dfk = -dFk - Real(2) * C.c * (Real(1) - xk);
-                if (m_abs(fk) <= Real(32) * RealLimits<Real>::eps() * (m_abs(Fk) + C.c * (Real(1) - xk) * (Real(1) - xk))) {
-                    conv = true;
-                    break;
-                }
+    }
+    if (series_step<Real, NSMAX>(C, x0, h, f0, df0, bm, R)) return true;
+    // near the root: when one Newton step puts x_eq within both bending
+    // scales of x0, a few Newton steps find it (f is smooth there) and the
+    // linearised solution about it finishes the cell
+    const Real est = df0 < Real(0) ? m_abs(f0 / df0) : RealLimits<Real>::inf();
+    const Real lim = C.b0 > Real(0) ? IntCfg<Real>::davg() : (-h * df0 > Real(50) ? IntCfg<Real>::drel() : IntCfg<Real>::zlin());
+    if (bm * est <= lim && est <= lim * (Real(1) - x0 + est)) {
+        Real xk = x0, fk = f0, dfk = df0, Fk = F0;
+        bool conv = false;
+        for (int it = 0; it < 4 && dfk < Real(0); it++) {
+            xk = m_min(m_max(xk - fk / dfk, Real(0)), Real(1));
+            Real dFk;
+            ode_F<Real, NSMAX>(C, xk, &Fk, &dFk);
+            fk = -Fk + C.c * (Real(1) - xk) * (Real(1) - xk);
+            dfk = -dFk - Real(2) * C.c * (Real(1) - xk);
+            if (m_abs(fk) <= Real(32) * RealLimits<Real>::eps() * (m_abs(Fk) + C.c * (Real(1) - xk) * (Real(1) - xk))) {
+                conv = true;
+                break;
             }
-            if (conv) {
-                SrcEq<Real> Q[NSMAX];
-                Real Dinf, bmax;
-                root_slope<Real, NSMAX>(C, xk, sigma0, Q, Dinf, bmax);
-                if (near_root_solution<Real>(C, xk, x0 - xk, Dinf, bmax, h, R)) return true;
-                R.x = x0;          // not close enough: leave it to the general part
-                R.IR = Real(0);
-            }
+        }
+        if (conv) {
+            // the slope at the root is the last one of the Newton steps
+            if (near_root_solution<Real>(C, xk, x0 - xk, -dfk, bm, h, R)) return true;
+            R.x = x0;          // not close enough: leave it to the general part
+            R.IR = Real(0);
         }
     }
     return false;
@@ -491,7 +594,7 @@ OOTS_HD IntResult<Real> integrate_general(const CellODE<Real> &C, Real x0, Real 
                                           Real F0, Real dF0, Real f0, const Eval &ev)
 {
     constexpr int G = IntCfg<Real>::G;
-    const Real xe = ev.template root<Real, NSMAX>(C, x0, f0, F0, dF0);
+    const Real xe = ev.template root<Real, NSMAX>(C, x0, f0, F0, dF0, sigma0);
     Real d0 = x0 - xe;
     if (d0 == Real(0)) {
         R.IR = h * C.c * (Real(1) - x0) * (Real(1) - x0);
