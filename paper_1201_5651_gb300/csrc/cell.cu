@@ -226,7 +226,10 @@ __global__ void __launch_bounds__(BS, 1024 / BS) cell_kernel(const GridDev<Real>
             if (m) {
                 const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
                 unsigned base = 0;
-                if (lane == leader) base = atomicAdd(qcount + (OP == OP_HALF ? 0 : 1), (unsigned)__popc(m));
+                if (lane == leader) {
+                    base = atomicAdd(qcount + (OP == OP_HALF ? 0 : 1), (unsigned)__popc(m));
+                    atomicAdd(&st->nq[OP == OP_HALF ? 0 : 1], (unsigned)__popc(m));
+                }
                 base = __shfl_sync(0xffffffffu, base, leader);
                 if (defer) {
                     const unsigned slot = base + __popc(m & ((1u << lane) - 1u));
@@ -269,6 +272,15 @@ __global__ void __launch_bounds__(BS, 1024 / BS) cell_kernel(const GridDev<Real>
     }
 }
 
+// Queued cells of a grid from which the general pass gives each of them one
+// thread (cell_seq_kernel) instead of a lane group.  By the grid's own count,
+// so that a grid takes the same path, and the same rounding, in any batch.
+// Measured in FP32, lane groups against threads (us): 16 k cells 69 / 170,
+// 46 k 92 / 115, 112 k 313 / 170, 162 k with many sources 1283 / 381.  In FP64
+// groups win at 9 k cells (2.9 ms / 5.5 ms: few warps, and a warp waits for
+// the longest of its cells in every loop) and no measured queue is longer.
+template <typename Real> __host__ __device__ constexpr unsigned seq_cells() { return 65536u; }
+
 // General pass: one lane group per queued cell (a half warp in FP32, a warp
 // in FP64; HALF: queue 0, FULL: queue 1).  Groups take the next queued cell
 // from a head counter (qcount[2 + queue]), so the pass ends when the cells
@@ -294,11 +306,29 @@ cell_general_kernel(const GridDev<Real> *grids, int ngrid, const long long *offs
     }
     const int qi = OP == OP_HALF ? 0 : 1;
     const unsigned nq = qcount[qi];
+    // with one grid, or few cells, every queued cell or none is this kernel's; otherwise a group
+    // claims as many cells as it has lanes and works through its own among them
+    const bool mixed = ngrid > 1 && nq >= seq_cells<Real>();
+    if (!mixed && nq >= seq_cells<Real>()) return;
+    unsigned todo = 0u, q0 = 0u;
     for (;;) {
         unsigned q = 0;
-        if (lane == 0) q = atomicAdd(&qcount[2 + qi], 1u);
-        q = __shfl_sync(gmask, q, gbase);
-        if (q >= nq) break;
+        if (mixed) {
+            while (todo == 0u) {
+                if (lane == 0) q0 = atomicAdd(&qcount[2 + qi], (unsigned)W);
+                q0 = __shfl_sync(gmask, q0, gbase);
+                if (q0 >= nq) break;
+                const bool own = q0 + lane < nq && grids[find_grid(offsets, ngrid, queue[q0 + lane])].st->nq[qi] < seq_cells<Real>();
+                todo = __ballot_sync(gmask, own) >> gbase;
+            }
+            if (todo == 0u) break;
+            q = q0 + __ffs(todo) - 1;
+            todo &= todo - 1u;
+        } else {
+            if (lane == 0) q = atomicAdd(&qcount[2 + qi], 1u);
+            q = __shfl_sync(gmask, q, gbase);
+            if (q >= nq) break;
+        }
         const long long idx = queue[q];
         const int gi = find_grid(offsets, ngrid, idx);
         const GridDev<Real> &G = grids[gi];
@@ -746,7 +776,10 @@ __global__ void __launch_bounds__(BS, (sizeof(Real) == 4 ? 1024 : 512) / BS) cel
             if (m) {
                 const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
                 unsigned qb = 0;
-                if (lane == leader) qb = atomicAdd(qcount + (OP == OP_HALF ? 0 : 1), (unsigned)__popc(m));
+                if (lane == leader) {
+                    qb = atomicAdd(qcount + (OP == OP_HALF ? 0 : 1), (unsigned)__popc(m));
+                    atomicAdd(&st->nq[OP == OP_HALF ? 0 : 1], (unsigned)__popc(m));
+                }
                 qb = __shfl_sync(0xffffffffu, qb, leader);
                 if (defer) queue[qb + __popc(m & ((1u << lane) - 1u))] = (unsigned)idx;
             }
@@ -804,11 +837,29 @@ cell_multi_general_kernel(const GridDev<Real> *grids, int ngrid, const long long
     }
     const int qi = OP == OP_HALF ? 0 : 1;
     const unsigned nq = qcount[qi];
+    // with one grid, or few cells, every queued cell or none is this kernel's; otherwise a group
+    // claims as many cells as it has lanes and works through its own among them
+    const bool mixed = ngrid > 1 && nq >= seq_cells<Real>();
+    if (!mixed && nq >= seq_cells<Real>()) return;
+    unsigned todo = 0u, q0 = 0u;
     for (;;) {
         unsigned q = 0;
-        if (lane == 0) q = atomicAdd(&qcount[2 + qi], 1u);
-        q = __shfl_sync(gmask, q, gbase);
-        if (q >= nq) break;
+        if (mixed) {
+            while (todo == 0u) {
+                if (lane == 0) q0 = atomicAdd(&qcount[2 + qi], (unsigned)W);
+                q0 = __shfl_sync(gmask, q0, gbase);
+                if (q0 >= nq) break;
+                const bool own = q0 + lane < nq && grids[find_grid(offsets, ngrid, queue[q0 + lane])].st->nq[qi] < seq_cells<Real>();
+                todo = __ballot_sync(gmask, own) >> gbase;
+            }
+            if (todo == 0u) break;
+            q = q0 + __ffs(todo) - 1;
+            todo &= todo - 1u;
+        } else {
+            if (lane == 0) q = atomicAdd(&qcount[2 + qi], 1u);
+            q = __shfl_sync(gmask, q, gbase);
+            if (q >= nq) break;
+        }
         const long long idx = queue[q];
         const int gi = find_grid(offsets, ngrid, idx);
         const GridDev<Real> &G = grids[gi];
@@ -867,6 +918,91 @@ cell_multi_general_kernel(const GridDev<Real> *grids, int ngrid, const long long
     }
 }
 
+// General pass for long queues: one thread per queued cell (NSMAX = 1: from
+// the closed-form pass's record; MAX_SRC: sources selected again).  A lane
+// group repeats the root search, the inversion and all scalar work of a cell
+// in every lane; with enough cells for the threads of the chip, a thread per
+// cell does that work once.
+template <typename Real, int OP, int NSMAX>
+__global__ void __launch_bounds__(128, sizeof(Real) == 4 ? 5 : 3)
+cell_seq_kernel(const GridDev<Real> *grids, int ngrid, const long long *offsets, const DevTable<Real> *tabs,
+                const unsigned *queue, unsigned *qcount, const Real *qrec)
+{
+    const int qi = OP == OP_HALF ? 0 : 1, lane = threadIdx.x & 31;
+    const unsigned nq = qcount[qi];
+    if (nq < seq_cells<Real>()) return;              // the lane groups take it
+    for (;;) {
+        unsigned q = 0;
+        if (lane == 0) q = atomicAdd(&qcount[4 + qi], 32u);
+        q = __shfl_sync(0xffffffffu, q, 0);
+        if (q >= nq) break;
+        q += lane;
+        double ions = 0.0, rec = 0.0;
+        int gi = -1;
+        const long long idx = q < nq ? queue[q] : 0;
+        if (q < nq) gi = find_grid(offsets, ngrid, idx);
+        if (gi >= 0 && grids[gi].st->nq[qi] < seq_cells<Real>()) gi = -1;   // a lane group's cell
+        if (gi >= 0) {
+            const GridDev<Real> &G = grids[gi];
+            DevState *st = G.st;
+            const long long g = idx - offsets[gi];
+            const Real h = Real(OP == OP_HALF ? 0.5 * st->dt : st->dt);
+            SrcRate<Real> r[NSMAX];
+            CellODE<Real> C;
+            Real n, x0, F0, dF0, f0;
+            IntResult<Real> R;
+            bool done = false;
+            if (NSMAX == 1) {
+                const Real *rv = qrec + (size_t)q * QREC;
+                x0 = rv[0]; n = rv[1];
+                r[0].A = rv[2]; r[0].b = rv[3]; r[0].Nin = rv[4]; r[0].p = rv[5]; r[0].tab = G.tab[0];
+                F0 = rv[6]; dF0 = rv[7]; f0 = rv[8];
+                C.ns = 1;
+                R.x = x0; R.IR = Real(0); R.lnfav = Real(0);
+            } else {
+                const int X = (int)(g % G.nx), Y = (int)((g / G.nx) % G.ny), Z = (int)(g / ((long long)G.nx * G.ny));
+                n = G.n ? G.n[g] : G.n_uniform;
+                x0 = G.x[g];
+                const SrcSel<Real> *sel = G.sel + (OP == OP_HALF ? 1 : 2) * MAX_SRC;
+                C.ns = gather_rates_sel<Real, NSMAX>(G, sel, OP == OP_FULL2 ? G.N2 : G.N1, tabs, X, Y, Z, g, n,
+                                                     st->lnthr[OP == OP_HALF ? 1 : 2], r);
+            }
+            C.c = G.alpha * n;
+            C.b0 = Real(0);
+            C.r = r;
+            C.tabs = tabs;
+            if (NSMAX != 1) done = integrate_prelude<Real, NSMAX>(C, x0, h, G.sigma0, R, F0, dF0, f0);
+            if (!done) R = integrate_general<Real, NSMAX>(C, x0, h, G.sigma0, R, F0, dF0, f0, SeqEval());
+            if (OP == OP_HALF) {
+                const_cast<Real *>(G.xh)[g] = R.x;
+            } else {
+                G.xout[g] = R.x;
+                const double nV = double(n) * st->cell_volume;
+                ions = nV * (double(x0) - double(R.x));
+                rec = nV * double(R.IR);
+            }
+        }
+        if (OP != OP_HALF) {
+            // budget: one set of atomics per warp where its cells lie in one grid
+            const int g0 = __reduce_max_sync(0xffffffffu, gi);
+            if (__all_sync(0xffffffffu, gi == g0 || gi < 0)) {
+                gi = g0;
+                for (int o = 16; o > 0; o >>= 1) {
+                    ions += __shfl_down_sync(0xffffffffu, ions, o);
+                    rec += __shfl_down_sync(0xffffffffu, rec, o);
+                }
+                if (lane != 0) gi = -1;
+            }
+            if (gi >= 0) {
+                DevState *st = grids[gi].st;
+                atomicAdd(&st->bud_step[1], ions + rec);
+                atomicAdd(&st->bud_step[2], ions);
+                atomicAdd(&st->bud_step[3], rec);
+            }
+        }
+    }
+}
+
 // stage 0: choose dt (Eq. 4 minimum or fixed, capped at t_end - t) and reset the step budget
 // stage 1: close the substep (t += dt, totals, done flag)
 template <typename Real>
@@ -874,7 +1010,7 @@ __global__ void finalize_kernel(const GridDev<Real> *grids, int ngrid, int stage
                                 const DevTable<Real> *tabs)
 {
     const int gi = blockIdx.x * blockDim.x + threadIdx.x;
-    if (stage == 0 && gi == 0) { qcount[0] = 0u; qcount[1] = 0u; qcount[2] = 0u; qcount[3] = 0u; }
+    if (stage == 0 && gi == 0) for (int q = 0; q < 6; q++) qcount[q] = 0u;
     if (gi >= ngrid) return;
     DevState *st = grids[gi].st;
     if (stage == 0) {
@@ -907,6 +1043,7 @@ __global__ void finalize_kernel(const GridDev<Real> *grids, int ngrid, int stage
                 G.sel[2 * MAX_SRC + s].nst = negligible_column<Real>(G, tabs, s, st->lnthr[2]);
             }
         }
+        st->nq[0] = st->nq[1] = 0u;
         st->bud_step[0] = st->sumQ * dt;
         st->bud_step[1] = st->bud_step[2] = st->bud_step[3] = 0.0;
     } else {
@@ -926,14 +1063,25 @@ static cudaError_t launch_cell_ns(const GridDev<Real> *grids, int ngrid, const l
 {
     const long long nb = (total + BS - 1) / BS;
     const int gbs = 256;                 // the general pass's blocks
+    const bool seq = total >= (long long)seq_cells<Real>();   // its queue may be long enough for a thread per cell
+    const int seq_blocks = gen_blocks * (sizeof(Real) == 4 ? 2 : 3);
     switch (op) {
     case OP_RATEDT: cell_kernel<Real, OP_RATEDT, NSMAX, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, qrec, rcache, use_cache); break;
     case OP_HALF: cell_kernel<Real, OP_HALF, NSMAX, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, qrec, rcache, use_cache); break;
     case OP_FULL1: cell_kernel<Real, OP_FULL1, NSMAX, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, qrec, rcache, use_cache); break;
     case OP_FULL2: cell_kernel<Real, OP_FULL2, NSMAX, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, qrec, rcache, use_cache); break;
-    case OP_HALF | OP_GENERAL: cell_general_kernel<Real, OP_HALF, NSMAX><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec); break;
-    case OP_FULL1 | OP_GENERAL: cell_general_kernel<Real, OP_FULL1, NSMAX><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec); break;
-    case OP_FULL2 | OP_GENERAL: cell_general_kernel<Real, OP_FULL2, NSMAX><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec); break;
+    case OP_HALF | OP_GENERAL:
+        if (seq) cell_seq_kernel<Real, OP_HALF, NSMAX><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
+        cell_general_kernel<Real, OP_HALF, NSMAX><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
+        break;
+    case OP_FULL1 | OP_GENERAL:
+        if (seq) cell_seq_kernel<Real, OP_FULL1, NSMAX><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
+        cell_general_kernel<Real, OP_FULL1, NSMAX><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
+        break;
+    case OP_FULL2 | OP_GENERAL:
+        if (seq) cell_seq_kernel<Real, OP_FULL2, NSMAX><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
+        cell_general_kernel<Real, OP_FULL2, NSMAX><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
+        break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -946,6 +1094,8 @@ static cudaError_t launch_cell_multi(const GridDev<Real> *grids, int ngrid, cons
 {
     const long long nb = (total + BS - 1) / BS;
     const int gbs = 256;                 // the general pass's blocks
+    const bool seq = total >= (long long)seq_cells<Real>();   // its queue may be long enough for a thread per cell
+    const int seq_blocks = gen_blocks * (sizeof(Real) == 4 ? 2 : 3);
     switch (op) {
     case OP_RATEDT:
         cell_multi_kernel<Real, OP_RATEDT, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 0);
@@ -957,9 +1107,18 @@ static cudaError_t launch_cell_multi(const GridDev<Real> *grids, int ngrid, cons
     case OP_HALF: cell_multi_kernel<Real, OP_HALF, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 0); break;
     case OP_FULL1: cell_multi_kernel<Real, OP_FULL1, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 0); break;
     case OP_FULL2: cell_multi_kernel<Real, OP_FULL2, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 0); break;
-    case OP_HALF | OP_GENERAL: cell_multi_general_kernel<Real, OP_HALF><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount); break;
-    case OP_FULL1 | OP_GENERAL: cell_multi_general_kernel<Real, OP_FULL1><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount); break;
-    case OP_FULL2 | OP_GENERAL: cell_multi_general_kernel<Real, OP_FULL2><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount); break;
+    case OP_HALF | OP_GENERAL:
+        if (seq) cell_seq_kernel<Real, OP_HALF, MAX_SRC><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, nullptr);
+        cell_multi_general_kernel<Real, OP_HALF><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount);
+        break;
+    case OP_FULL1 | OP_GENERAL:
+        if (seq) cell_seq_kernel<Real, OP_FULL1, MAX_SRC><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, nullptr);
+        cell_multi_general_kernel<Real, OP_FULL1><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount);
+        break;
+    case OP_FULL2 | OP_GENERAL:
+        if (seq) cell_seq_kernel<Real, OP_FULL2, MAX_SRC><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, nullptr);
+        cell_multi_general_kernel<Real, OP_FULL2><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount);
+        break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -79,6 +79,7 @@ struct DevState {
     double bud_total[4];      // accumulated since the last reset
     double cell_volume;       // dx^3
     long long nsub;           // substeps taken
+    unsigned nq[2];           // cells of this grid left to the general pass: half step, full step
     int done;                 // t >= t_end
     int err;                  // DEVERR_*
     float lnthr[4];           // source-selection thresholds ln(1e-3 eps / H), set with each step: the next
