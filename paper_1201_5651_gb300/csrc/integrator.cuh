@@ -215,12 +215,12 @@ template <> struct IntCfg<float> {
     static OOTS_HD float zser() { return 0.2f; }
     static OOTS_HD float dser() { return 0.1f; }
     static OOTS_HD float drel() { return 2e-2f; }
-    static OOTS_HD float davg() { return 3e-4f; }
+    static OOTS_HD float davg() { return 1e-4f; }
 };
 
-template <typename Real, int NSMAX>
+template <typename Real, int NSMAX, typename Eval>
 OOTS_HD Real attenuation_average(const CellODE<Real> &C, const SrcEq<Real> *Q, Real xe, Real d0, Real Dinf,
-                                 Real h, Real ustar, Real ut, bool in_panels, Real wt);
+                                 Real h, Real ustar, Real ut, bool in_panels, const Eval &ev);
 
 // Root of the convex, decreasing right-hand side by Newton inside the
 // bracket [lo, hi], from xk (with f, F and f' there): from the right of the
@@ -290,9 +290,9 @@ struct SeqEval {
     }
 };
 #ifdef __CUDACC__
-template <int W> struct GroupEval {
+template <int W, bool ATT = false> struct GroupEval {
     static_assert(W == 16 || W == 32, "half warp or whole warp");
-    static constexpr bool attenuation = false;   // integration passes only (b0 = 0)
+    static constexpr bool attenuation = ATT;     // the integration passes have b0 = 0
     int lane;          // lane within the group, 0..W-1
     int base;          // first lane of the group within its warp
     unsigned mask;     // the group's lanes
@@ -778,7 +778,7 @@ OOTS_HD IntResult<Real> integrate_general(const CellODE<Real> &C, Real x0, Real 
     R.x = xe + d0 * m_exp(ustar);
     R.IR = IR;
     if (Eval::attenuation && C.b0 > Real(0))
-        R.lnfav = attenuation_average<Real, NSMAX>(C, Q, xe, d0, Dinf, h, ustar, ut, found, wt);
+        R.lnfav = attenuation_average<Real, NSMAX>(C, Q, xe, d0, Dinf, h, ustar, ut, found, ev);
     return R;
 }
 
@@ -799,9 +799,12 @@ OOTS_HD IntResult<Real> integrate_cell(const CellODE<Real> &C, Real x0, Real h, 
 // exp(-b0 (x - x_min)) is largest at that end and falls monotonically away
 // from it, so the integral is marched from the heavy end with adaptive panels
 // (relative to the sum so far) and stopped where the weight is negligible.
-template <typename Real, int NSMAX>
+// (Summed on the first pass's panels it is wrong for thick cells: those panels
+// do not know where the step will end, and the weight falls by e^-25 and more
+// between that point and the end of its panel.)
+template <typename Real, int NSMAX, typename Eval>
 OOTS_HD Real attenuation_average(const CellODE<Real> &C, const SrcEq<Real> *Q, Real xe, Real d0, Real Dinf,
-                                 Real h, Real ustar, Real ut, bool in_panels, Real wt)
+                                 Real h, Real ustar, Real ut, bool in_panels, const Eval &ev)
 {
     constexpr int G = IntCfg<Real>::G;
     const Real xend = xe + d0 * m_exp(ustar);
@@ -814,14 +817,14 @@ OOTS_HD Real attenuation_average(const CellODE<Real> &C, const SrcEq<Real> *Q, R
         const Real wte = m_exp(ut);
         const Real e0 = m_exp(-C.b0 * (xe - xmin));
         Real q[G], qt[G];
-#pragma unroll
-        for (int g = 0; g < G; g++) {
-            Real w = Real(0.5) * wte * (Real(1) + GL<G>::template x<Real>(g));
-            Real d = d0 * w;
-            Real invD = Real(1) / ode_D<Real, NSMAX>(C, Q, xe, d);
-            q[g] = (m_exp(-C.b0 * (xe + d - xmin)) * invD - e0 / Dinf) / w;
-            qt[g] = (invD - Real(1) / Dinf) / w;
-        }
+        auto node = [&](int l, Real &v) {
+            const Real w = Real(0.5) * wte * (Real(1) + GL<G>::template x<Real>(l));
+            const Real d = d0 * w;
+            const Real invD = Real(1) / ode_D<Real, NSMAX>(C, Q, xe, d);
+            v = (m_exp(-C.b0 * (xe + d - xmin)) * invD - e0 / Dinf) / w;
+            return (invD - Real(1) / Dinf) / w;
+        };
+        ev.template eval<G>(node, qt, q);
         Real cq[G], cqt[G];
         leg_coeffs<Real, G>(q, cq);
         leg_coeffs<Real, G>(qt, cqt);
@@ -846,21 +849,23 @@ OOTS_HD Real attenuation_average(const CellODE<Real> &C, const SrcEq<Real> *Q, R
         Real lo = m_min(pos, nxt), hi = m_max(pos, nxt);
         Real mid = Real(0.5) * (lo + hi), hw = Real(0.5) * (hi - lo);
         Real full = Real(0), halves = Real(0), thalves = Real(0);
+        // nodes 0 .. G-1 of the lower half, G .. 2G-1 of the upper one, 2G .. 3G-1 of the whole panel
+        Real iv[3 * G], wv[3 * G];
+        auto node = [&](int l, Real &v) {
+            const int part = l / G, g = l - part * G;
+            const Real m2 = part == 2 ? mid : mid + (part ? Real(0.5) : Real(-0.5)) * hw, w2 = part == 2 ? hw : Real(0.5) * hw;
+            const Real d = d0 * m_exp(m2 + w2 * GL<G>::template x<Real>(g));
+            const Real invD = Real(1) / ode_D<Real, NSMAX>(C, Q, xe, d);
+            v = m_exp(-C.b0 * (xe + d - xmin)) * invD;
+            return invD;
+        };
+        ev.template eval<3 * G>(node, iv, wv);
 #pragma unroll
         for (int g = 0; g < G; g++) {
-            Real d = d0 * m_exp(mid + hw * GL<G>::template x<Real>(g));
-            full += GL<G>::template w<Real>(g) * hw * m_exp(-C.b0 * (xe + d - xmin)) / ode_D<Real, NSMAX>(C, Q, xe, d);
-        }
-#pragma unroll
-        for (int hh = 0; hh < 2; hh++) {
-            Real m2 = mid + (hh ? Real(0.5) : Real(-0.5)) * hw;
-#pragma unroll
-            for (int g = 0; g < G; g++) {
-                Real d = d0 * m_exp(m2 + Real(0.5) * hw * GL<G>::template x<Real>(g));
-                Real invD = Real(1) / ode_D<Real, NSMAX>(C, Q, xe, d);
-                halves += GL<G>::template w<Real>(g) * Real(0.5) * hw * m_exp(-C.b0 * (xe + d - xmin)) * invD;
-                thalves += GL<G>::template w<Real>(g) * Real(0.5) * hw * invD;
-            }
+            const Real w = GL<G>::template w<Real>(g) * hw;
+            full += w * wv[2 * G + g];
+            halves += Real(0.5) * w * (wv[g] + wv[G + g]);
+            thalves += Real(0.5) * w * (iv[g] + iv[G + g]);
         }
         np++;
         if (m_abs(full - halves) > IntCfg<Real>::tolq() * Real(10) * (S + halves) && hw > Real(1e-12)) {

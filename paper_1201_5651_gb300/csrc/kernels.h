@@ -15,50 +15,13 @@ template <typename Real> struct DevTable;
 struct ff;
 template <typename Real> struct ColT;
 
-// Tile shapes of the implicit wavefront sweep (A1): (id, TX, TY, TZ); one chain
-// thread per (j,k) column (TY*TZ a multiple of 32) plus one producer warp.
-// Shapes with TY*TZ = 32 keep the whole plane chain in one warp.
-#define OOTS_SHAPES(X) \
-    X(0, 16, 8, 8)     \
-    X(1, 16, 8, 4)     \
-    X(2, 16, 16, 16)   \
-    X(3, 32, 8, 4)     \
-    X(4, 8, 8, 8)      \
-    X(5, 16, 16, 8)    \
-    X(6, 8, 8, 4)
-// Shapes 7 and 8 are other names of shapes 4 (8 x 8 x 8) and 0 (16 x 8 x 8).
-// The traces of the explicit schemes have no tiles: every shape runs the march.
-enum { NUM_SHAPES = 9, SHAPE_TP8 = 7, SHAPE_TP16 = 8 };
+// The tile shapes of oots_set_tile_shape.  The marches below have blocks of
+// their own, so the shapes only keep their meaning at the interface: dims, and
+// the one that FP64 refuses (its tile once needed more shared memory than a
+// block has).
+enum { NUM_SHAPES = 9, SHAPE_16_CUBED = 2 };
 static const int SHAPE_DIMS[NUM_SHAPES][3] = {{16, 8, 8}, {16, 8, 4}, {16, 16, 16}, {32, 8, 4}, {8, 8, 8},
                                               {16, 16, 8}, {8, 8, 4}, {8, 8, 8}, {16, 8, 8}};
-inline int sweep_twin(int shape) { return shape == SHAPE_TP8 ? 4 : (shape == SHAPE_TP16 ? 0 : shape); }
-
-template <typename Real> struct SweepParams {
-    const GridDev<Real> *grids;
-    const Job *jobs;
-    const TileItem *items;
-    int nitems;
-    unsigned *ticket;                  // zeroed before each launch
-    unsigned *done;                    // CTAs finished; zeroed before each launch
-    unsigned *epoch;                   // launches finished so far (persistent; starts at 0)
-    unsigned long long *faces;         // per tile 3 faces x FMAX cells x tagged words (zeroed once)
-    const DevTable<Real> *tabs;
-    int *err;                          // sticky device error
-    long long spin_limit;              // bounded wait on upstream tiles
-    long long skip_publish;            // tile that never writes its faces (fault-injection test), -1: none
-    int chunk;                         // planes per hand-off chunk (<= 0: 4)
-    int ngrid;                         // grids in `grids` (> 0: the launch returns at once when every
-                                       // grid has reached its end time; 0: no such check)
-};
-
-// tagged 8-byte words per published face cell (mixed path 3, FP64 path 4)
-template <typename Real> constexpr int face_words() { return sizeof(Real) == 4 ? 3 : 4; }
-
-template <typename Real> cudaError_t prepare_sweeps();
-template <typename Real> int sweep_occupancy(int shape);             // resident CTAs per SM
-template <typename Real> bool sweep_shape_ok(int shape);              // fits the shared memory of this device
-template <typename Real>
-cudaError_t launch_sweep(const SweepParams<Real> &P, int shape, int nblocks, cudaStream_t s);
 
 // The column march (march.cuh).  A published cell is one 16-byte record: its
 // outgoing column (float-float in the mixed path) and weight factor.
@@ -74,12 +37,14 @@ template <typename Real> struct MarchParams {
     int which;                         // 0: trace x into N1; 1: trace xh into N2
     unsigned *ticket, *done;           // zero before each launch (the launch leaves them so)
     unsigned *epoch;                   // launches finished so far (persistent; starts at 0)
+    const DevTable<Real> *tabs;        // A1
     MCell<Real> *halo;
-    unsigned *progress;                // per item: chunks of layers published, tagged with the launch's epoch
+    unsigned long long *progress;      // per item: chunks of layers published, tagged with the launch's epoch
     int *err;                          // sticky device error
     long long spin_limit;              // bounded wait on upstream items
     long long skip_publish;            // item that never publishes (fault-injection test), -1: none
-    int ngrid;                         // as SweepParams::ngrid
+    int ngrid;                         // grids in `grids` (> 0: the launch returns at once when every
+                                       // grid has reached its end time; 0: no such check)
     int narr;                          // input arrays of a cell: 1 (x or n x packed), 2 when some grid brings n and x
 };
 
@@ -89,6 +54,11 @@ template <typename Real> struct MarchShape { enum { NW = 7, RPT = sizeof(Real) =
 template <typename Real> cudaError_t march_occupancy(int narr, int *per_sm);
 template <typename Real>
 cudaError_t launch_march(const MarchParams<Real> &P, int nblocks, cudaStream_t s);
+// A1 (march_a1.cuh): blocks of 32 x kMarchA1Warps cells; reads the state from GridDev::xh, writes xout
+constexpr int kMarchA1Warps = 7;
+template <typename Real> cudaError_t march_a1_occupancy(int *per_sm);
+template <typename Real>
+cudaError_t launch_march_a1(const MarchParams<Real> &P, int nblocks, cudaStream_t s);
 // n x of the traced state (which = 0: x, 1: xh) into each grid's padded rows (GridDev::nxp);
 // max_elems = the largest grid's padded cells
 template <typename Real>
@@ -150,11 +120,11 @@ OOTS_HOSTDEV inline long long make_march_item(MarchItem &I, const March &M, int 
 // implicit = 1 runs the A1 row integration instead (single source).  The jobs
 // along x come first (nrow0 of them, threads0 threads); nthreads is the sum
 // of plane_job_threads over all jobs, whose `first` fields are the running
-// sums.
+// sums.  rows0: the first job's rows (A1's only source).
 long long plane_job_threads(int code, long long rows);
 template <typename Real>
 cudaError_t launch_plane(const GridDev<Real> *grids, const PlaneJob *jobs, int njobs, int nrow0, long long nthreads,
-                         long long threads0, const DevTable<Real> *tabs, int which, int implicit, cudaStream_t s);
+                         long long threads0, long long rows0, const DevTable<Real> *tabs, int which, int implicit, cudaStream_t s);
 
 // Per-cell passes.  HALF and FULL run as a closed-form pass over all cells
 // followed by the general pass (op | OP_GENERAL) over the queued cells.

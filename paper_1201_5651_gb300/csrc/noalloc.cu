@@ -192,8 +192,8 @@ int trace_noalloc(DevSetup &S, int nx, int ny, int nz, double dx, const void *n_
     // the per-item arrays after the fixed part: progress words first (they must
     // keep the tags of earlier launches, so their place does not move)
     size_t off = items_offset<double>();
-    unsigned *progress = (unsigned *)(sc + off);
-    off += kMaxItems * sizeof(unsigned);
+    unsigned long long *progress = (unsigned long long *)(sc + off);
+    off += kMaxItems * sizeof(unsigned long long);
     MarchItem *items = (MarchItem *)(sc + off);
     off += kMaxItems * sizeof(MarchItem);
     int *at = (int *)(sc + off);
@@ -214,6 +214,7 @@ int trace_noalloc(DevSetup &S, int nx, int ny, int nz, double dx, const void *n_
     P.ticket = (unsigned *)(sc + kOffTicket);
     P.done = (unsigned *)(sc + kOffTicket) + 1;
     P.epoch = (unsigned *)(sc + kOffEpoch);
+    P.tabs = nullptr;
     P.halo = halo;
     P.progress = progress;
     P.err = (int *)(sc + kOffErr);

@@ -147,24 +147,21 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
     int shape = 0;
     int scheme = OOTS_A3;
     GridDev<Real> *d_grids = nullptr;
-    Job *d_jobs = nullptr;
-    TileItem *d_items = nullptr;
-    int nitems = 0;
-    long long ntiles = 0;
-    unsigned *d_sync = nullptr;        // implicit sweep: [0] ticket, [1] done (zeroed per sweep), [16] epoch; march: [32], [33], [48]
-    unsigned long long *d_faces = nullptr;
-    March *d_marches = nullptr;        // column march: pyramids, items, published halos, progress per item
-    MarchItem *d_mitems = nullptr;
-    int nmitems = 0;
-    int mblocks = 1;
-    int narr = 1;                      // its input arrays: 2 when some grid brings n and x unpacked
-    MCell<Real> *d_halo = nullptr;
-    unsigned *d_progress = nullptr;
+    // march launches (0: traces, 1: A1): items, published halos, progress per item
+    struct MarchList {
+        MarchItem *items = nullptr;
+        int nitems = 0, blocks = 1;
+        MCell<Real> *halo = nullptr;
+        unsigned long long *progress = nullptr;
+    } ml[2];
+    March *d_marches = nullptr;        // pyramids of every point source
+    int narr = 1;                      // input arrays of a trace: 2 when some grid brings n and x unpacked
+    unsigned *d_sync = nullptr;        // per march list: ticket, finished CTAs; epoch 16 words on (kept by the launches)
     Real *d_nxp = nullptr;             // n x of the traced state, packed (grids with many sources)
     long long pack_max = 0;            // padded cells of the largest packed grid (0: none)
     PlaneJob *d_pjobs = nullptr;       // plane-parallel sources
     int npjobs = 0, nrow0 = 0;         // jobs; of them, rows along x (first in the array)
-    long long plane_threads = 0, threads0 = 0;
+    long long plane_threads = 0, threads0 = 0, plane_rows = 0;
     DevTable<Real> *d_tabs = nullptr;
     std::vector<void *> tabmem;
     long long *d_offsets = nullptr;
@@ -176,28 +173,25 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
     unsigned *d_qcount = nullptr;      // queue lengths of the half and full integrations
     int gen_blocks = 1;                // grid of the general pass
     int cell_bs = 128;                 // threads per block of the closed-form passes
-    int nblocks1 = 1;
     int nsmax = 1;                     // largest source count among the grids
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     bool graph_fixed = false;
     int *d_err = nullptr;
     long long spin_limit = 1ll << 22, skip_publish = -1;
-    int sweep_chunk = 0;
 
     ~LaunchSet() override
     {
         if (gexec) cudaGraphExecDestroy(gexec);
         if (graph) cudaGraphDestroy(graph);
         cudaFree(d_grids);
-        cudaFree(d_jobs);
-        cudaFree(d_items);
-        cudaFree(d_sync);
-        cudaFree(d_faces);
+        for (auto &m : ml) {
+            cudaFree(m.items);
+            cudaFree(m.halo);
+            cudaFree(m.progress);
+        }
         cudaFree(d_marches);
-        cudaFree(d_mitems);
-        cudaFree(d_halo);
-        cudaFree(d_progress);
+        cudaFree(d_sync);
         cudaFree(d_nxp);
         cudaFree(d_pjobs);
         cudaFree(d_tabs);
@@ -245,23 +239,17 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
         device = c0->device;
         scheme = c0->scheme;
         shape = shape_req >= 0 ? shape_req : 0;
-        if (!sweep_shape_ok<Real>(shape))
+        if (shape == SHAPE_16_CUBED && sizeof(Real) == 8)
             return fail(OOTS_E_UNSUPPORTED, "tile shape %d does not fit in shared memory at this precision", shape);
         d_err = c0->d_err;
         spin_limit = c0->spin_limit;
         skip_publish = c0->skip_publish;
-        sweep_chunk = c0->sweep_chunk;
-        const int TX = SHAPE_DIMS[shape][0], TY = SHAPE_DIMS[shape][1], TZ = SHAPE_DIMS[shape][2];
-        const int T3[3] = {TX, TY, TZ};
-        const int FMAX = std::max(TY * TZ, std::max(TX * TZ, TX * TY));
 
         std::vector<GridDev<Real>> grids(cs.size());
-        std::vector<Job> jobs;
         std::vector<PlaneJob> pjobs;
-        std::vector<TileItem> items;
         std::vector<DevTable<Real>> tabs;
         std::vector<long long> offs(cs.size());
-        long long tile_base = 0, off = 0;
+        long long off = 0;
         std::vector<March> marches;
         std::vector<long long> pack_base(cs.size(), -1);
         long long packed = 0;
@@ -329,8 +317,7 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
                     pjobs.push_back(P);
                     continue;
                 }
-                // (A1 traces only for a criterion on dx/dt)
-                for (int o = 0; o < 8 && (scheme != OOTS_A1 || c->crit.K3 > 0 || c->crit.K4 > 0); o++)
+                for (int o = 0; o < 8; o++)
                     for (int a = 0; a < 3; a++) {
                         March M;
                         if (!make_march(M, c->nx, c->ny, c->nz, S.v, o, a, G.pitch, pack_base[g] >= 0)) continue;
@@ -339,49 +326,11 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
                         M.src = s;
                         marches.push_back(M);
                     }
-                if (scheme != OOTS_A1) continue;
-                for (int o = 0; o < 8; o++) {
-                    Job J;
-                    memset(&J, 0, sizeof(J));
-                    J.grid = (int)g;
-                    J.src = s;
-                    bool empty = false;
-                    for (int a = 0; a < 3; a++) {
-                        J.v[a] = S.v[a];
-                        J.sg[a] = (o >> a) & 1 ? -1 : 1;
-                        J.ext[a] = J.sg[a] > 0 ? n3[a] - S.v[a] : S.v[a];
-                        if (J.ext[a] <= 0) empty = true;
-                        const int r = S.v[a] % T3[a];
-                        J.off[a] = c->tile_align ? 0 : (J.sg[a] > 0 ? r : (T3[a] - r) % T3[a]);
-                        J.nt[a] = (J.ext[a] + J.off[a] + T3[a] - 1) / T3[a];
-                    }
-                    if (empty) continue;
-                    J.tile_base = tile_base;
-                    const int jid = (int)jobs.size();
-                    for (int K = 0; K < J.nt[2]; K++)
-                        for (int Jj = 0; Jj < J.nt[1]; Jj++)
-                            for (int I = 0; I < J.nt[0]; I++) {
-                                TileItem t;
-                                t.job = jid;
-                                t.I = (unsigned short)I;
-                                t.J = (unsigned short)Jj;
-                                t.K = (unsigned short)K;
-                                t.pad = 0;
-                                items.push_back(t);
-                            }
-                    tile_base += (long long)J.nt[0] * J.nt[1] * J.nt[2];
-                    jobs.push_back(J);
-                }
             }
             offs[g] = off;
             off += c->ncell;
         }
         total = off;
-        ntiles = tile_base;
-        nitems = (int)items.size();
-        std::stable_sort(items.begin(), items.end(), [](const TileItem &a, const TileItem &b) {
-            return a.I + a.J + a.K < b.I + b.J + b.K;
-        });
 
         CU(cudaSetDevice(device));
         if (packed > 0) {
@@ -432,23 +381,21 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
         CU(cudaMalloc(&d_rcache, (size_t)std::max(total, 1ll) * 3 * sizeof(Real)));
         CU(cudaMalloc(&d_qcount, 8 * sizeof(unsigned)));
         CU(cudaMemset(d_qcount, 0, 8 * sizeof(unsigned)));
-        if (!marches.empty() || !jobs.empty()) {
+        if (!marches.empty()) {
             CU(cudaMalloc(&d_sync, 256));
             CU(cudaMemset(d_sync, 0, 256));
-        }
-        if (!marches.empty()) {
-            int rc = build_march(marches, c0->nsm);
-            if (rc) return rc;
-        }
-        if (!jobs.empty()) {
-            CU(cudaMalloc(&d_jobs, jobs.size() * sizeof(Job)));
-            CU(cudaMemcpy(d_jobs, jobs.data(), jobs.size() * sizeof(Job), cudaMemcpyHostToDevice));
-            CU(cudaMalloc(&d_items, items.size() * sizeof(TileItem)));
-            CU(cudaMemcpy(d_items, items.data(), items.size() * sizeof(TileItem), cudaMemcpyHostToDevice));
-            // faces start with epoch 0 in every word; launches use epochs 1, 2, ...
-            const size_t fbytes = (size_t)ntiles * 3 * FMAX * face_words<Real>() * sizeof(unsigned long long);
-            CU(cudaMalloc(&d_faces, fbytes));
-            CU(cudaMemset(d_faces, 0, fbytes));
+            CU(cudaMalloc(&d_marches, marches.size() * sizeof(March)));
+            CU(cudaMemcpy(d_marches, marches.data(), marches.size() * sizeof(March), cudaMemcpyHostToDevice));
+            int rc = OOTS_OK, per_sm = 0;
+            // (A1 traces only for a criterion on dx/dt)
+            if (scheme != OOTS_A1 || c0->crit.K3 > 0 || c0->crit.K4 > 0) {
+                CU(march_occupancy<Real>(narr, &per_sm));
+                if ((rc = build_march(ml[0], marches, MarchShape<Real>::ROWS, per_sm * c0->nsm))) return rc;
+            }
+            if (scheme == OOTS_A1) {
+                CU(march_a1_occupancy<Real>(&per_sm));
+                if ((rc = build_march(ml[1], marches, kMarchA1Warps, per_sm * c0->nsm))) return rc;
+            }
         }
         if (!pjobs.empty()) {
             // rows along x first (their trace kernel differs), then the rest
@@ -463,14 +410,13 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
             CU(cudaMalloc(&d_pjobs, pjobs.size() * sizeof(PlaneJob)));
             CU(cudaMemcpy(d_pjobs, pjobs.data(), pjobs.size() * sizeof(PlaneJob), cudaMemcpyHostToDevice));
             npjobs = (int)pjobs.size();
+            plane_rows = pjobs[0].rows;
         }
         if (!tabs.empty()) {
             CU(cudaMalloc(&d_tabs, tabs.size() * sizeof(DevTable<Real>)));
             CU(cudaMemcpy(d_tabs, tabs.data(), tabs.size() * sizeof(DevTable<Real>), cudaMemcpyHostToDevice));
         }
-        if (scheme == OOTS_A1) CU(prepare_sweeps<Real>());
         int nsm = c0->nsm;
-        if (scheme == OOTS_A1) nblocks1 = sweep_occupancy<Real>(shape) * nsm;
         gen_blocks = cell_general_occupancy<Real>(nsmax) * nsm;
         // closed-form passes: 128-thread blocks for many sources (a slow cell holds up fewer others),
         // 256 for one source (cheap cells; fewer block set-ups), unless tuned
@@ -480,9 +426,8 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
 
     // The march's work list: the blocks of every pyramid, handed out in order of
     // T1 + T2 (an item's upstream blocks come first), longer ones first among equals.
-    int build_march(const std::vector<March> &marches, int nsm)
+    int build_march(MarchList &L, const std::vector<March> &marches, int rows, int blocks)
     {
-        const int rows = MarchShape<Real>::ROWS;
         std::vector<MarchItem> list;
         std::vector<long long> first(marches.size()), pubs;
         for (size_t m = 0; m < marches.size(); m++) {
@@ -518,33 +463,31 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
             cells += pubs[order[i]];
             items[i] = I;
         }
-        nmitems = (int)items.size();
-        CU(cudaMalloc(&d_marches, marches.size() * sizeof(March)));
-        CU(cudaMemcpy(d_marches, marches.data(), marches.size() * sizeof(March), cudaMemcpyHostToDevice));
-        CU(cudaMalloc(&d_mitems, items.size() * sizeof(MarchItem)));
-        CU(cudaMemcpy(d_mitems, items.data(), items.size() * sizeof(MarchItem), cudaMemcpyHostToDevice));
-        CU(cudaMalloc(&d_halo, (size_t)std::max(cells, 1ll) * sizeof(MCell<Real>)));
-        CU(cudaMalloc(&d_progress, items.size() * sizeof(unsigned)));
-        CU(cudaMemset(d_progress, 0, items.size() * sizeof(unsigned)));
-        int per_sm = 0;
-        CU(march_occupancy<Real>(narr, &per_sm));
-        mblocks = per_sm * nsm;
+        L.nitems = (int)items.size();
+        L.blocks = blocks;
+        CU(cudaMalloc(&L.items, items.size() * sizeof(MarchItem)));
+        CU(cudaMemcpy(L.items, items.data(), items.size() * sizeof(MarchItem), cudaMemcpyHostToDevice));
+        CU(cudaMalloc(&L.halo, (size_t)std::max(cells, 1ll) * sizeof(MCell<Real>)));
+        CU(cudaMalloc(&L.progress, items.size() * sizeof(unsigned long long)));
+        CU(cudaMemset(L.progress, 0, items.size() * sizeof(unsigned long long)));
         return OOTS_OK;
     }
 
-    MarchParams<Real> march_params(int which) const
+    MarchParams<Real> march_params(int list, int which) const
     {
+        const MarchList &L = ml[list];
         MarchParams<Real> P;
         P.grids = d_grids;
         P.marches = d_marches;
-        P.items = d_mitems;
-        P.nitems = nmitems;
+        P.items = L.items;
+        P.nitems = L.nitems;
         P.which = which;
-        P.ticket = d_sync + 32;
-        P.done = d_sync + 33;
-        P.epoch = d_sync + 48;
-        P.halo = d_halo;
-        P.progress = d_progress;
+        P.ticket = d_sync + 32 * list;
+        P.done = d_sync + 32 * list + 1;
+        P.epoch = d_sync + 32 * list + 16;
+        P.tabs = d_tabs;
+        P.halo = L.halo;
+        P.progress = L.progress;
         P.err = d_err;
         P.spin_limit = spin_limit;
         P.skip_publish = skip_publish;
@@ -553,31 +496,11 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
         return P;
     }
 
-    SweepParams<Real> params() const
-    {
-        SweepParams<Real> P;
-        P.grids = d_grids;
-        P.jobs = d_jobs;
-        P.items = d_items;
-        P.nitems = nitems;
-        P.ticket = d_sync;
-        P.done = d_sync + 1;
-        P.epoch = d_sync + 16;
-        P.faces = d_faces;
-        P.tabs = d_tabs;
-        P.err = d_err;
-        P.spin_limit = spin_limit;
-        P.skip_publish = skip_publish;
-        P.chunk = sweep_chunk;
-        P.ngrid = (int)ctxs.size();
-        return P;
-    }
-
     // trace (mode 0) or A1 implicit sweep (mode 1) of every source: point
     // sources by the wavefront sweep, plane sources row by row
     int sweep(cudaStream_t s, int which, int mode)
     {
-        if (mode == 0 && nmitems > 0) {
+        if (mode == 0 && ml[0].nitems > 0) {
             if (prof) prof->mark(0);
             if (pack_max > 0) {
                 // the trace's input packed
@@ -585,18 +508,20 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
                 if (prof) prof->mark(OOTS_K_PACK);
                 if (prof) prof->mark(0);
             }
-            CU(launch_march<Real>(march_params(which), mblocks, s));
+            CU(launch_march<Real>(march_params(0, which), ml[0].blocks, s));
             if (prof) prof->mark(which == 0 ? OOTS_K_SWEEP1 : OOTS_K_SWEEP2);
         }
-        if (mode == 1 && nitems > 0) {
-            CU(cudaMemsetAsync(d_sync, 0, 2 * sizeof(unsigned), s));   // ticket and done; the epoch persists
+        if (mode == 1 && ml[1].nitems > 0) {
+            // (A1 runs one grid) the state as the march reads it, while it writes x
+            oots_ctx *c = ctxs[0];
+            CU(cudaMemcpyAsync(c->d_xh, c->d_x, (size_t)c->ncell * sizeof(Real), cudaMemcpyDeviceToDevice, s));
             if (prof) prof->mark(0);
-            CU(launch_sweep<Real>(params(), shape, nblocks1, s));
+            CU(launch_march_a1<Real>(march_params(1, 0), ml[1].blocks, s));
             if (prof) prof->mark(OOTS_K_IMPLICIT);
         }
         if (npjobs > 0) {
             if (prof) prof->mark(0);
-            CU(launch_plane<Real>(d_grids, d_pjobs, npjobs, nrow0, plane_threads, threads0, d_tabs, which, mode, s));
+            CU(launch_plane<Real>(d_grids, d_pjobs, npjobs, nrow0, plane_threads, threads0, plane_rows, d_tabs, which, mode, s));
             if (prof) prof->mark(mode == 1 ? OOTS_K_PLANE_IMPLICIT : OOTS_K_PLANE_TRACE);
         }
         return OOTS_OK;

@@ -9,19 +9,6 @@ enum { MAX_SRC = 64 };          // sources per grid
 // Device-side error codes written to DevState::err (first one sticks).
 enum { DEVERR_NONE = 0, DEVERR_TIMEOUT = 1, DEVERR_BOUNDS = 2 };
 
-// One (grid, source, octant) sweep: the octant of cells on one side of the
-// source vertex along each axis, traced outward from the vertex (Sect. 5).
-struct Job {
-    int grid;              // index into the launch's grid array
-    int src;               // source index within the grid
-    int v[3];              // source vertex
-    int sg[3];             // octant signs (+1 / -1)
-    int ext[3];            // octant extent in cells
-    int off[3];            // tile offset: octant-local i of tile I starts at I*T - off
-    int nt[3];             // tiles per axis
-    long long tile_base;   // index of tile (0,0,0) in the flag and face arrays
-};
-
 // One plane-parallel source of one grid (a source at infinity whose rays run
 // along a grid axis, Sect. 3.1): its rows are traced independently (the
 // thread layout per axis is in plane.cu).
@@ -33,9 +20,6 @@ struct PlaneJob {
     long long rows;        // rows of cells parallel to the axis
     long long first;       // first thread of the job in the launch (a multiple of 256)
 };
-
-// One tile of a job, ordered in the work list by tile diagonal I+J+K.
-struct TileItem { int job; unsigned short I, J, K, pad; };
 
 // One pyramid of the column march (march.cuh): the cells of one octant of one
 // source whose dominant axis is `axis`, layer l of that axis holding the cells

@@ -221,18 +221,20 @@ __global__ void __launch_bounds__(256, ROWX ? 3 : 2) plane_trace_kernel(const Gr
     }
 }
 
-// A1 with a plane source: one thread per row integrates its cells in the
-// direction of travel; photon budget by warp sums, one atomic per warp.
-template <typename Real>
+// A1 with a plane source: W threads per row integrate its cells in the
+// direction of travel; photon budget by warp sums, one atomic per warp.  W = 1
+// when rows fill the chip; otherwise a lane group per row, which repeats the
+// scalar work of a cell in every lane and spreads the quadrature nodes of the
+// cells no closed form settles, so that a row's chain of cells is shorter.
+template <typename Real, int W>
 __global__ void __launch_bounds__(128) plane_implicit_kernel(const GridDev<Real> *grids, const PlaneJob *jobs,
-                                                             int njobs, long long nthreads,
                                                              const DevTable<Real> *tabs)
 {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t - (threadIdx.x & 31) >= nthreads) return;
-    const PlaneJob J = jobs[find_plane_job(jobs, njobs, t - (threadIdx.x & 31))];
+    const PlaneJob J = jobs[0];                      // A1 takes a single source
     const GridDev<Real> &G = grids[J.grid];
-    const long long r = t - J.first;
+    const long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / W;
+    const int lane32 = threadIdx.x & 31, base = lane32 & ~(W - 1), lane = lane32 - base;
+    const unsigned gmask = W == 32 ? 0xffffffffu : ((1u << (W & 31)) - 1u) << base;
     double ions = 0.0, rec = 0.0;
     const Real dt = Real(G.st->dt);
     if (r < J.rows) {
@@ -250,12 +252,20 @@ __global__ void __launch_bounds__(128) plane_implicit_kernel(const GridDev<Real>
             src_rate<Real>(rt, G.qfac[s], G.tab[s], sig, G.dx, n, true, 0, 0, 0, Real(N), tabs);
             CellODE<Real> C;
             C.ns = 1; C.c = G.alpha * n; C.b0 = sig * n * G.dx; C.r = &rt; C.tabs = tabs;
-            const IntResult<Real> Rs = integrate_cell<Real, 1>(C, x0, dt, sig);
+            IntResult<Real> Rs;
+            if constexpr (W == 1) {
+                Rs = integrate_cell<Real, 1>(C, x0, dt, sig);
+            } else {
+                __syncwarp(gmask);                   // every lane has read x0 before lane 0 writes x
+                Real F0, dF0, f0;
+                if (!integrate_prelude<Real, 1>(C, x0, dt, sig, Rs, F0, dF0, f0))
+                    Rs = integrate_general<Real, 1>(C, x0, dt, sig, Rs, F0, dF0, f0, GroupEval<W, true>{lane, base, gmask});
+            }
             Real dtau_eff = -Rs.lnfav;
             if (!(dtau_eff >= Real(0))) dtau_eff = Real(0);
-            N1[g] = Real(N);
+            if (lane == 0) N1[g] = Real(N);
             N += double(dtau_eff) / double(sig);
-            if (dt > Real(0)) {
+            if (dt > Real(0) && lane == 0) {
                 G.xout[g] = Rs.x;
                 const double nV = double(n) * cellV;
                 ions += nV * double(x0 - Rs.x);
@@ -275,6 +285,9 @@ __global__ void __launch_bounds__(128) plane_implicit_kernel(const GridDev<Real>
     }
 }
 
+// rows up to which A1 gives each a lane group
+constexpr long long kGroupRows = 4096;
+
 long long plane_job_threads(int code, long long rows)
 {
     // axis 0: a warp per row; axes 1, 2: 256 threads per 32 rows.  Whole
@@ -285,13 +298,16 @@ long long plane_job_threads(int code, long long rows)
 
 template <typename Real>
 cudaError_t launch_plane(const GridDev<Real> *grids, const PlaneJob *jobs, int njobs, int nrow0, long long nthreads,
-                         long long threads0, const DevTable<Real> *tabs, int which, int implicit, cudaStream_t s)
+                         long long threads0, long long rows0, const DevTable<Real> *tabs, int which, int implicit, cudaStream_t s)
 {
     if (njobs <= 0 || nthreads <= 0) return cudaSuccess;
     if (implicit) {
         const int bs = 128;
-        plane_implicit_kernel<Real><<<(unsigned)((nthreads + bs - 1) / bs), bs, 0, s>>>(grids, jobs, njobs, nthreads,
-                                                                                        tabs);
+        constexpr int W = GroupWidth<Real>::value;
+        if (rows0 <= kGroupRows)
+            plane_implicit_kernel<Real, W><<<(unsigned)((rows0 * W + bs - 1) / bs), bs, 0, s>>>(grids, jobs, tabs);
+        else
+            plane_implicit_kernel<Real, 1><<<(unsigned)((rows0 + bs - 1) / bs), bs, 0, s>>>(grids, jobs, tabs);
         return cudaGetLastError();
     }
     const int bs = 256;
@@ -304,9 +320,9 @@ cudaError_t launch_plane(const GridDev<Real> *grids, const PlaneJob *jobs, int n
     return cudaGetLastError();
 }
 
-template cudaError_t launch_plane<double>(const GridDev<double> *, const PlaneJob *, int, int, long long, long long,
+template cudaError_t launch_plane<double>(const GridDev<double> *, const PlaneJob *, int, int, long long, long long, long long,
                                           const DevTable<double> *, int, int, cudaStream_t);
-template cudaError_t launch_plane<float>(const GridDev<float> *, const PlaneJob *, int, int, long long, long long,
+template cudaError_t launch_plane<float>(const GridDev<float> *, const PlaneJob *, int, int, long long, long long, long long,
                                          const DevTable<float> *, int, int, cudaStream_t);
 
 } // namespace oots

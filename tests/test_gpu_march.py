@@ -55,3 +55,32 @@ def test_packed_columns_and_repeated_traces(precision, nx, nsrc):
                 assert _rel(got[s], P.trace(s, w.x0)) <= TOL[precision], s
         else:
             assert all(np.array_equal(a, b) for a, b in zip(first, got))
+
+
+@pytest.mark.parametrize("dims,pos,spectrum", [
+    ((33, 9, 15), (0, 0, 0), "mono"), ((7, 34, 8), (3, 34, 4), "bb"), ((14, 15, 32), (14, 0, 16), "mono"), ((1, 9, 1), (0, 4, 0), "bb"),
+])
+def test_a1_at_block_edges_fp64(dims, pos, spectrum):
+    """A1 (blocks of 32 x 7 cells, a hand-off per layer): state and entry columns after one step against the
+    oracle.  1e-9 as every FP64 step: cells integrate to 1e-13 there and here, columns sum ~40 of them."""
+    w = inputs.small_random(n=dims[0], ny=dims[1], nz=dims[2], seed=3 + sum(dims), nsrc=1, spectrum=spectrum)
+    w.sources[0].pos = tuple(float(p) for p in pos)
+    d = 0.05 * w.t_rec
+    c = oots.Context.from_workload(w, "fp64", scheme=oots.OOTS_A1, dt_fixed=d)
+    c.step(d)
+    x = np.ascontiguousarray(w.x0.astype(np.float64))
+    _, _, bud, _ = oracle.Problem.from_workload(w).substep(x, 0.0, d, scheme=1, dt_fixed=d)
+    assert float(np.max(np.abs(c.get_neutral_fraction() - x))) <= 1e-9
+    assert np.allclose(c.get_budget(), bud, rtol=1e-8)      # tied cells are counted once
+
+
+@pytest.mark.parametrize("ny,nz", [(60, 66), (72, 65)])
+def test_a1_plane_rows_on_both_sides_of_the_group_rule(ny, nz):
+    """3960 rows take a lane group each, 4680 a thread each: both follow the oracle (1e-9, as above)."""
+    w = inputs.plane_random(n=6, ny=ny, nz=nz, seed=8, axis=0, x_lo=0.2)
+    d = 0.02 * w.t_rec
+    c = oots.Context.from_workload(w, "fp64", scheme=oots.OOTS_A1, dt_fixed=d)
+    c.step(d)
+    x = np.ascontiguousarray(w.x0.astype(np.float64))
+    oracle.Problem.from_workload(w).substep(x, 0.0, d, scheme=1, dt_fixed=d)
+    assert float(np.max(np.abs(c.get_neutral_fraction() - x))) <= 1e-9
