@@ -7,10 +7,10 @@
 // The integrations run in two passes.  The first pass settles every cell that
 // a closed form covers (photon-free, at its root, or slow enough for the
 // linearised step: almost all of them) and appends the others to a queue.
-// The second pass gives each queued cell a whole warp: the quadrature nodes
+// The second pass gives each queued cell a lane group: the quadrature nodes
 // of every panel are evaluated one per lane, so the few slow cells near the
 // ionisation front neither hold up warps of fast cells nor run their node
-// evaluations one after another.
+// evaluations one after another.  A long queue goes a thread per cell instead.
 #include <algorithm>
 
 #include "common.cuh"
@@ -46,21 +46,16 @@ __device__ __forceinline__ bool cells_live(const GridDev<Real> *grids, int lo, i
     return false;
 }
 
-// Rate parameters of every source for the cell at global index g = (X,Y,Z).
-// with_p = false leaves r[s].p of tabulated sources to the caller.
-template <typename Real, int NSMAX>
-__device__ __forceinline__ int cell_rates(const GridDev<Real> &G, const Real *Ncol, const DevTable<Real> *tabs,
-                                          int X, int Y, int Z, long long g, Real n, SrcRate<Real> *r,
-                                          bool with_p = true)
+// Octant-local indices of a cell from source vertex v.
+__device__ __forceinline__ int oct_index(int X, int v) { return X >= v ? X - v : v - 1 - X; }
+
+// Coordinates of cell g of a grid (below 2^32 cells, so 32-bit divisions).
+__device__ __forceinline__ void cell_xyz(unsigned g, unsigned nx, unsigned nxy, int &X, int &Y, int &Z)
 {
-    for (int s = 0; s < NSMAX && s < G.nsrc; s++) {
-        const int i = X >= G.vtx[s][0] ? X - G.vtx[s][0] : G.vtx[s][0] - 1 - X;
-        const int j = Y >= G.vtx[s][1] ? Y - G.vtx[s][1] : G.vtx[s][1] - 1 - Y;
-        const int k = Z >= G.vtx[s][2] ? Z - G.vtx[s][2] : G.vtx[s][2] - 1 - Z;
-        src_rate<Real>(r[s], G.qfac[s], G.tab[s], G.sigma0, G.dx, n, G.pcode[s] != 0, i, j, k,
-                       Ncol[(long long)s * G.ncell + g], tabs, with_p);
-    }
-    return G.nsrc;
+    const unsigned z = g / nxy, rem = g - z * nxy, y = rem / nx;
+    Z = (int)z;
+    Y = (int)y;
+    X = (int)(rem - y * nx);
 }
 
 // Mixed path: warp sums of two FP32 values, scaled to FP64 once per warp,
@@ -81,6 +76,15 @@ __device__ __forceinline__ void block_sum2_f(float a, float b, double scale, dou
     }
 }
 
+// s + e += v, the rounding error of s collected in e: a thread's budget over
+// the cells of its run, no less exact than one cell's.
+__device__ __forceinline__ void add_two(float &s, float &e, float v)
+{
+    const float t = __fadd_rn(s, v), w = __fsub_rn(t, s);
+    e += __fadd_rn(__fsub_rn(s, __fsub_rn(t, w)), __fsub_rn(v, w));
+    s = t;
+}
+
 // Block sums of two values in one pass (one pair of barriers); thread 0 gets both.
 __device__ __forceinline__ void block_sum2(double &a, double &b, double *sh)
 {
@@ -98,35 +102,71 @@ __device__ __forceinline__ void block_sum2(double &a, double &b, double *sh)
     }
 }
 
-template <typename Real, int OP, int NSMAX, int BS>
-__global__ void __launch_bounds__(BS, 1024 / BS) cell_kernel(const GridDev<Real> *grids, int ngrid, const long long *offsets,
+// Block minimum of the Eq. 4 step into the grid's state.
+template <typename Real>
+__device__ __forceinline__ void block_dtmin(double dtmin, float dtmin_f, DevState *st, double *sh)
+{
+    if (sizeof(Real) == 4) {
+        for (int o = 16; o > 0; o >>= 1) dtmin_f = fminf(dtmin_f, __shfl_down_sync(0xffffffffu, dtmin_f, o));
+        if ((threadIdx.x & 31) == 0) dtmin = double(dtmin_f);   // lane 0 carries the warp minimum
+    } else {
+        for (int o = 16; o > 0; o >>= 1) dtmin = fmin(dtmin, __shfl_down_sync(0xffffffffu, dtmin, o));
+    }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __syncthreads();
+    if (lane == 0) sh[wid] = dtmin;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double m = sh[0];
+        for (int w = 1; w < (int)(blockDim.x >> 5); w++) m = fmin(m, sh[w]);
+        // (the read skips the atomic of a block that cannot lower the minimum)
+        const unsigned long long mb = (unsigned long long)__double_as_longlong(m);
+        if (m < 1e300 && mb < *(volatile unsigned long long *)&st->dt_bits) atomicMin(&st->dt_bits, mb);
+    }
+}
+
+// Closed-form pass of grids with one source.  A block takes a run of `run`
+// consecutive cells (a multiple of BS): locating its grid, the step and the
+// reductions are done once per run and grid, not once per BS cells, and the
+// cells of a run are addressed with 32-bit arithmetic.  (A block per BS cells
+// was bound by that prologue, a chain of dependent loads and two barriers, and
+// by 64-bit divisions.)  What bounds it now is instruction issue: at 256^3 with
+// a monochromatic source the dt pass moves 400 MB in 163 us (about a third of
+// the copy rate) and the full step 268 us.  Measured before and after, the runs
+// and the fused table evaluation (tab_all) together, us: 256^3 monochromatic,
+// dt / half / full 430 / 391 / 555 -> 163 / 256 / 268; 256^3 blackbody plane
+// 610 / 582 / 1200 -> 376 / 432 / 786; 128^3 blackbody 84 / 55 / 112 ->
+// 51 / 45 / 80; 64^3 in FP64 (bound by the FP64 pipe) 205 / 203 / 395 ->
+// 168 / 230 / 395.  FP64 takes 128 registers a thread: at 64 its spills cost
+// more than the second half of the warps gave (half step 230 against 315 us).
+template <typename Real, int OP, int BS>
+__global__ void __launch_bounds__(BS, (sizeof(Real) == 4 ? 1024 : 512) / BS) cell_kernel(const GridDev<Real> *grids, int ngrid, const long long *offsets,
                                                    long long total, const DevTable<Real> *tabs, unsigned *queue,
-                                                   unsigned *qcount, Real *qrec, Real *rcache, int use_cache)
+                                                   unsigned *qcount, Real *qrec, Real *rcache, int use_cache, int run)
 {
     __shared__ double sh[32];
     __shared__ int s_grid_lo, s_grid_hi;
-    const long long base = (long long)blockIdx.x * blockDim.x;
-    // every thread of a block works on one grid at a time; a block straddling
-    // two grids loops over both (the reductions are per grid)
+    const long long run_lo = (long long)blockIdx.x * run, run_hi = run_lo + run < total ? run_lo + run : total;
+    // every thread of a block works on one grid at a time; a run over several
+    // grids loops over them (the reductions are per grid)
     if (threadIdx.x == 0) {
-        long long last = base + blockDim.x - 1;
-        if (last >= total) last = total - 1;
-        s_grid_lo = find_grid(offsets, ngrid, base < total ? base : total - 1);
-        s_grid_hi = find_grid(offsets, ngrid, last);
+        s_grid_lo = find_grid(offsets, ngrid, run_lo);
+        s_grid_hi = find_grid(offsets, ngrid, run_hi - 1);
         if (!cells_live<Real, OP>(grids, s_grid_lo, s_grid_hi)) s_grid_hi = s_grid_lo - 1;
     }
     __syncthreads();
     // mixed path: the step and the Eq. 4 factors in FP32, converted once per
-    // block (this GPU runs FP64 at a small fraction of its FP32 rate, so the
-    // per-cell criterion and budget stay off the FP64 pipe)
+    // run and grid (this GPU runs FP64 at a small fraction of its FP32 rate, so
+    // the per-cell criterion and budget stay off the FP64 pipe)
     constexpr bool F32 = sizeof(Real) == 4;
     __shared__ float s_f[4];
     for (int gi = s_grid_lo; gi <= s_grid_hi; gi++) {
         const GridDev<Real> &G = grids[gi];
         DevState *st = G.st;
-        const long long idx = base + threadIdx.x;
-        const bool mine = idx < total && idx >= offsets[gi] && (gi + 1 >= ngrid || idx < offsets[gi + 1]) &&
-                          idx - offsets[gi] >= G.cell_lo && idx - offsets[gi] < G.cell_hi;
+        const long long off = offsets[gi], gend = gi + 1 < ngrid ? offsets[gi + 1] : total;
+        // this grid's cells of the run: cnt of them from lo (none of a stopped grid)
+        const long long clo = max(max(run_lo, off) - off, G.cell_lo), chi = min(min(run_hi, gend) - off, G.cell_hi);
+        const unsigned lo = (unsigned)clo;
         if (F32) {
             if (threadIdx.x == 0) {
                 const double d = st->dt;
@@ -139,128 +179,138 @@ __global__ void __launch_bounds__(BS, 1024 / BS) cell_kernel(const GridDev<Real>
         }
         const double dtd = F32 ? 0.0 : st->dt;
         const bool stepping = F32 ? s_f[0] > 0.0f : dtd > 0.0;
-        const bool active = mine && (OP == OP_RATEDT || stepping) && !(OP == OP_RATEDT && st->done);
+        const bool live = OP == OP_RATEDT ? !st->done : stepping;
+        const int cnt = live && chi > clo ? (int)(chi - clo) : 0;
         double dtmin = __longlong_as_double(0x7ff0000000000000ll);
         float dtmin_f = __int_as_float(0x7f800000);
         double ions = 0.0, rec = 0.0;
-        float ions_f = 0.0f, rec_f = 0.0f;
-        bool defer = false;
-        Real rv[QREC];
-        if (active) {
-            const long long g = idx - offsets[gi];
-            const int X = (int)(g % G.nx);
-            const int Y = (int)((g / G.nx) % G.ny);
-            const int Z = (int)(g / ((long long)G.nx * G.ny));
-            const Real n = G.n ? G.n[g] : G.n_uniform;
-            const Real x0 = G.x[g];
-            SrcRate<Real> r[NSMAX];
-            const Real *Ncol = (OP == OP_FULL2) ? G.N2 : G.N1;
-            CellODE<Real> C;
-            // single source, same state and columns as this substep's dt pass:
-            // its transmitted fraction and F, F' at x0 come from the rate cache
-            const bool cached = NSMAX == 1 && (OP == OP_HALF || OP == OP_FULL1) && use_cache;
-            C.ns = cell_rates<Real, NSMAX>(G, Ncol, tabs, X, Y, Z, g, n, r, !cached);
-            if (cached && C.ns > 0) r[0].p = rcache[idx];
-            C.c = G.alpha * n;
-            C.b0 = Real(0);
-            C.r = r;
-            C.tabs = tabs;
-            if (OP == OP_RATEDT) {
-                // Eq. 4 with T fixed: K1 t_rec, K3 max(0.05, x)/|dx/dt|, K4/|dx/dt|
-                Real F, dF;
-                ode_F<Real, NSMAX>(C, x0, &F, &dF);
-                if (NSMAX == 1 && rcache && C.ns > 0) {
-                    rcache[idx] = r[0].p;
-                    rcache[total + idx] = F;
-                    rcache[2 * total + idx] = dF;
+        float ions_f = 0.0f, rec_f = 0.0f, ions_e = 0.0f, rec_e = 0.0f;
+        const unsigned nx = (unsigned)G.nx, nxy = (unsigned)G.nx * (unsigned)G.ny;
+        const bool lit = G.nsrc > 0, plane = G.pcode[0] != 0;
+        const int tab = G.tab[0], v0 = G.vtx[0][0], v1 = G.vtx[0][1], v2 = G.vtx[0][2];
+        const Real qfac = G.qfac[0], sigma0 = G.sigma0, dx = G.dx, alpha = G.alpha, nu = G.n_uniform;
+        const Real *xs = G.x;
+        const Real *__restrict__ nd = G.n;
+        const Real *__restrict__ Ncol = (OP == OP_FULL2) ? G.N2 : G.N1;
+        // same state and columns as this substep's dt pass: its transmitted
+        // fraction and F, F' at x0 come from the rate cache
+        const bool cached = (OP == OP_HALF || OP == OP_FULL1) && use_cache && lit;
+        Real *cache = rcache + off;
+        Real x0n = Real(0), nn = nu, Nn = Real(0);
+        int o = threadIdx.x;
+        if (o < cnt) {
+            const unsigned g = lo + o;
+            x0n = xs[g];
+            if (nd) nn = nd[g];
+            if (lit) Nn = Ncol[g];
+        }
+        for (int o0 = 0; o0 < cnt; o0 += BS, o += BS) {
+            const bool active = o < cnt;
+            const unsigned g = lo + o;
+            const Real x0 = x0n, n = nn, N = Nn;
+            // the next cell's loads run under this one's arithmetic
+            if (o + BS < cnt) {
+                x0n = xs[g + BS];
+                if (nd) nn = nd[g + BS];
+                if (lit) Nn = Ncol[g + BS];
+            }
+            bool defer = false;
+            Real rv[QREC];
+            if (active) {
+                int X, Y, Z;
+                cell_xyz(g, nx, nxy, X, Y, Z);
+                SrcRate<Real> r;
+                CellODE<Real> C;
+                C.ns = lit ? 1 : 0;
+                C.c = alpha * n;
+                C.b0 = Real(0);
+                C.r = &r;
+                C.tabs = tabs;
+                Real F = Real(0), dF = Real(0);
+                const int i = oct_index(X, v0), j = oct_index(Y, v1), k = oct_index(Z, v2);
+                if (cached) {
+                    src_rate<Real>(r, qfac, tab, sigma0, dx, n, plane, i, j, k, N, tabs, false);
+                    r.p = cache[g];
+                    F = cache[total + g];
+                    dF = cache[2 * total + g];
+                } else if (lit) {
+                    src_rate_F<Real>(r, qfac, tab, sigma0, dx, n, plane, i, j, k, N, tabs, x0, F, dF);
                 }
-                if (F32) {
-                    const float xd = fabsf(float(-F + C.c * (Real(1) - x0) * (Real(1) - x0)));
-                    if (s_f[1] > 0.0f) dtmin_f = fminf(dtmin_f, s_f[1] / (float(G.alpha) * float(n)));
-                    if (xd > 0.0f) {
-                        if (s_f[2] > 0.0f) dtmin_f = fminf(dtmin_f, s_f[2] * fmaxf(0.05f, float(x0)) / xd);
-                        if (s_f[3] > 0.0f) dtmin_f = fminf(dtmin_f, s_f[3] / xd);
+                if (OP == OP_RATEDT) {
+                    // Eq. 4 with T fixed: K1 t_rec, K3 max(0.05, x)/|dx/dt|, K4/|dx/dt|
+                    if (rcache && lit) {
+                        cache[g] = r.p;
+                        cache[total + g] = F;
+                        cache[2 * total + g] = dF;
                     }
-                } else {
-                    const double xd = fabs((double)(-F + C.c * (Real(1) - x0) * (Real(1) - x0)));
-                    if (st->K1 > 0) dtmin = fmin(dtmin, st->K1 / (double(G.alpha) * double(n)));
-                    if (xd > 0) {
-                        if (st->K3 > 0) dtmin = fmin(dtmin, st->K3 * fmax(0.05, (double)x0) / xd);
-                        if (st->K4 > 0) dtmin = fmin(dtmin, st->K4 / xd);
-                    }
-                }
-            } else {
-                // closed forms here; the rest goes to the warp-per-cell pass
-                IntResult<Real> R;
-                Real F0 = Real(0), dF0 = Real(0), f0;
-                const Real h = F32 ? Real(s_f[0]) : Real(OP == OP_HALF ? 0.5 * dtd : dtd);
-                if (cached && C.ns > 0) { F0 = rcache[total + idx]; dF0 = rcache[2 * total + idx]; }
-                if (integrate_prelude<Real, NSMAX>(C, x0, h, G.sigma0, R, F0, dF0, f0, cached && C.ns > 0)) {
-                    if (OP == OP_HALF) {
-                        const_cast<Real *>(G.xh)[g] = R.x;
+                    if (F32) {
+                        const float xd = fabsf(float(-F + C.c * (Real(1) - x0) * (Real(1) - x0)));
+                        if (s_f[1] > 0.0f) dtmin_f = fminf(dtmin_f, s_f[1] / (float(alpha) * float(n)));
+                        if (xd > 0.0f) {
+                            if (s_f[2] > 0.0f) dtmin_f = fminf(dtmin_f, s_f[2] * fmaxf(0.05f, float(x0)) / xd);
+                            if (s_f[3] > 0.0f) dtmin_f = fminf(dtmin_f, s_f[3] / xd);
+                        }
                     } else {
-                        G.xout[g] = R.x;
-                        if (F32) {
-                            // per H atom times n; the cell volume is applied per warp
-                            ions_f = float(n) * (float(x0) - float(R.x));
-                            rec_f = float(n) * float(R.IR);
-                        } else {
-                            const double nV = double(n) * st->cell_volume;
-                            ions = nV * (double(x0) - double(R.x));
-                            rec = nV * double(R.IR);
+                        const double xd = fabs((double)(-F + C.c * (Real(1) - x0) * (Real(1) - x0)));
+                        if (st->K1 > 0) dtmin = fmin(dtmin, st->K1 / (double(alpha) * double(n)));
+                        if (xd > 0) {
+                            if (st->K3 > 0) dtmin = fmin(dtmin, st->K3 * fmax(0.05, (double)x0) / xd);
+                            if (st->K4 > 0) dtmin = fmin(dtmin, st->K4 / xd);
                         }
                     }
                 } else {
-                    defer = true;
-                    if (NSMAX == 1) {
+                    // closed forms here; the rest goes to the general pass
+                    IntResult<Real> R;
+                    Real f0;
+                    const Real h = F32 ? Real(s_f[0]) : Real(OP == OP_HALF ? 0.5 * dtd : dtd);
+                    if (integrate_prelude<Real, 1>(C, x0, h, sigma0, R, F, dF, f0, lit)) {
+                        if (OP == OP_HALF) {
+                            const_cast<Real *>(G.xh)[g] = R.x;
+                        } else {
+                            G.xout[g] = R.x;
+                            if (F32) {
+                                // per H atom times n; the cell volume is applied per warp
+                                add_two(ions_f, ions_e, float(n) * (float(x0) - float(R.x)));
+                                add_two(rec_f, rec_e, float(n) * float(R.IR));
+                            } else {
+                                const double nV = double(n) * st->cell_volume;
+                                ions += nV * (double(x0) - double(R.x));
+                                rec += nV * double(R.IR);
+                            }
+                        }
+                    } else {
+                        defer = true;
                         // what the general pass would otherwise recompute
-                        rv[0] = x0; rv[1] = n; rv[2] = r[0].A; rv[3] = r[0].b; rv[4] = r[0].Nin; rv[5] = r[0].p;
-                        rv[6] = F0; rv[7] = dF0; rv[8] = f0;
+                        rv[0] = x0; rv[1] = n; rv[2] = r.A; rv[3] = r.b; rv[4] = r.Nin; rv[5] = r.p;
+                        rv[6] = F; rv[7] = dF; rv[8] = f0;
                     }
                 }
             }
-        }
-        if (OP != OP_RATEDT) {
-            // warp-aggregated append to the queue of the general pass
-            const unsigned m = __ballot_sync(0xffffffffu, defer);
-            if (m) {
-                const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
-                unsigned base = 0;
-                if (lane == leader) {
-                    base = atomicAdd(qcount + (OP == OP_HALF ? 0 : 1), (unsigned)__popc(m));
-                    atomicAdd(&st->nq[OP == OP_HALF ? 0 : 1], (unsigned)__popc(m));
-                }
-                base = __shfl_sync(0xffffffffu, base, leader);
-                if (defer) {
-                    const unsigned slot = base + __popc(m & ((1u << lane) - 1u));
-                    queue[slot] = (unsigned)idx;
-                    if (NSMAX == 1)
+            if (OP != OP_RATEDT) {
+                // warp-aggregated append to the queue of the general pass
+                const unsigned m = __ballot_sync(0xffffffffu, defer);
+                if (m) {
+                    const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
+                    unsigned qb = 0;
+                    if (lane == leader) {
+                        qb = atomicAdd(qcount + (OP == OP_HALF ? 0 : 1), (unsigned)__popc(m));
+                        atomicAdd(&st->nq[OP == OP_HALF ? 0 : 1], (unsigned)__popc(m));
+                    }
+                    qb = __shfl_sync(0xffffffffu, qb, leader);
+                    if (defer) {
+                        const unsigned slot = qb + __popc(m & ((1u << lane) - 1u));
+                        queue[slot] = (unsigned)(off + g);
 #pragma unroll
                         for (int v = 0; v < QREC; v++) qrec[(size_t)slot * QREC + v] = rv[v];
+                    }
                 }
             }
         }
         if (OP == OP_RATEDT) {
-            if (F32) {
-                for (int o = 16; o > 0; o >>= 1) dtmin_f = fminf(dtmin_f, __shfl_down_sync(0xffffffffu, dtmin_f, o));
-                if ((threadIdx.x & 31) == 0) dtmin = double(dtmin_f);   // lane 0 carries the warp minimum
-            } else {
-                for (int o = 16; o > 0; o >>= 1) dtmin = fmin(dtmin, __shfl_down_sync(0xffffffffu, dtmin, o));
-            }
-            const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-            __syncthreads();
-            if (lane == 0) sh[wid] = dtmin;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double m = sh[0];
-                for (int w = 1; w < (int)(blockDim.x >> 5); w++) m = fmin(m, sh[w]);
-                // (the read skips the atomic of a block that cannot lower the minimum)
-                const unsigned long long mb = (unsigned long long)__double_as_longlong(m);
-                if (m < 1e300 && mb < *(volatile unsigned long long *)&st->dt_bits) atomicMin(&st->dt_bits, mb);
-            }
+            block_dtmin<Real>(dtmin, dtmin_f, st, sh);
         } else if (OP == OP_FULL1 || OP == OP_FULL2) {
             double si = ions, sr = rec;
-            if (F32) block_sum2_f(ions_f, rec_f, st->cell_volume, si, sr, sh);
+            if (F32) block_sum2_f(ions_f + ions_e, rec_f + rec_e, st->cell_volume, si, sr, sh);
             else block_sum2(si, sr, sh);
             if (threadIdx.x == 0 && (si != 0.0 || sr != 0.0)) {
                 atomicAdd(&st->bud_step[1], si + sr);   // absorbed = new ions + recombinations
@@ -289,7 +339,7 @@ template <typename Real> __host__ __device__ constexpr unsigned seq_cells() { re
 // quadrature nodes are spread over the lanes (WarpEval).  Budget sums of FULL
 // are gathered per block in shared memory for up to eight grids and flushed
 // with one atomic per grid and block.
-template <typename Real, int OP, int NSMAX>
+template <typename Real, int OP>
 __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 4 : 2)
 cell_general_kernel(const GridDev<Real> *grids, int ngrid, const long long *offsets, const DevTable<Real> *tabs,
                     const unsigned *queue, unsigned *qcount, const Real *qrec)
@@ -335,36 +385,21 @@ cell_general_kernel(const GridDev<Real> *grids, int ngrid, const long long *offs
         DevState *st = G.st;
         const double dtd = st->dt;
         const long long g = idx - offsets[gi];
-        SrcRate<Real> r[NSMAX];
+        // the closed-form pass left the cell's rates and f(x0)
+        SrcRate<Real> r[1];
         CellODE<Real> C;
-        Real n, x0, F0, dF0, f0;
         IntResult<Real> R;
         const Real h = Real(OP == OP_HALF ? 0.5 * dtd : dtd);
-        bool done = false;
-        if (NSMAX == 1) {
-            // one source: the closed-form pass left its rates and f(x0)
-            const Real *rv = qrec + (size_t)q * QREC;
-            x0 = rv[0]; n = rv[1];
-            r[0].A = rv[2]; r[0].b = rv[3]; r[0].Nin = rv[4]; r[0].p = rv[5]; r[0].tab = G.tab[0];
-            F0 = rv[6]; dF0 = rv[7]; f0 = rv[8];
-            C.ns = 1;
-            R.x = x0; R.IR = Real(0); R.lnfav = Real(0);
-        } else {
-            const int X = (int)(g % G.nx);
-            const int Y = (int)((g / G.nx) % G.ny);
-            const int Z = (int)(g / ((long long)G.nx * G.ny));
-            n = G.n ? G.n[g] : G.n_uniform;
-            x0 = G.x[g];
-            const Real *Ncol = (OP == OP_FULL2) ? G.N2 : G.N1;
-            C.ns = cell_rates<Real, NSMAX>(G, Ncol, tabs, X, Y, Z, g, n, r);
-        }
+        const Real *rv = qrec + (size_t)q * QREC;
+        const Real x0 = rv[0], n = rv[1];
+        r[0].A = rv[2]; r[0].b = rv[3]; r[0].Nin = rv[4]; r[0].p = rv[5]; r[0].tab = G.tab[0];
+        C.ns = 1;
         C.c = G.alpha * n;
         C.b0 = Real(0);
         C.r = r;
         C.tabs = tabs;
-        if (NSMAX != 1) done = integrate_prelude<Real, NSMAX>(C, x0, h, G.sigma0, R, F0, dF0, f0);
-        if (!done)
-            R = integrate_general<Real, NSMAX>(C, x0, h, G.sigma0, R, F0, dF0, f0, GroupEval<W>{lane, gbase, gmask});
+        R.x = x0; R.IR = Real(0); R.lnfav = Real(0);
+        R = integrate_general<Real, 1>(C, x0, h, G.sigma0, R, rv[6], rv[7], rv[8], GroupEval<W>{lane, gbase, gmask});
         if (lane == 0) {
             if (OP == OP_HALF) {
                 const_cast<Real *>(G.xh)[g] = R.x;
@@ -474,20 +509,20 @@ __device__ __forceinline__ void load_columns8(const GridDev<Real> &G, const Real
     for (int q = 0; q < 8; q++) Nb[q] = s0 + q < G.nsrc ? Ncol[(long long)(s0 + q) * G.ncell + g] : Real(0);
 }
 
-// Rate parameters of the sources whose bound exceeds e^lnthr, into
-// r[0 .. NK-1] (indices fixed at compile time, so r stays in registers).
-// Returns how many there are; NK + 1 when there are more than NK.  sel: the
-// pass's source records; a source whose entry column is at or beyond its
-// record's negligible column is left out without forming its bound.
-template <typename Real, int NK>
-__device__ __forceinline__ int gather_rates_sel(const GridDev<Real> &G, const SrcSel<Real> *sel, const Real *Ncol,
-                                                const DevTable<Real> *tabs, int X, int Y, int Z, long long g, Real n,
-                                                float lnthr, SrcRate<Real> *r)
+// The sources whose bound at cell g exceeds e^lnthr, as a bit mask; ampsum:
+// plus the sum of their bounds.  sel: the pass's source records; a source whose
+// entry column is at or beyond its record's negligible column is left out
+// without forming its bound.
+template <typename Real, bool SUM>
+__device__ __forceinline__ unsigned long long select_sources(const GridDev<Real> &G, const SrcSel<Real> *sel, const Real *Ncol,
+                                                             int X, int Y, int Z, long long g, float lnthr, float &ampsum)
 {
-    int cnt = 0;
+    static_assert(MAX_SRC <= 64, "one bit per source");
+    unsigned long long mask = 0;
     for (int s0 = 0; s0 < G.nsrc; s0 += 8) {
         Real Nb[8];
         load_columns8(G, Ncol, s0, g, Nb);
+        unsigned m = 0;
 #pragma unroll
         for (int q = 0; q < 8; q++) {
             const int s = s0 + q;
@@ -496,21 +531,60 @@ __device__ __forceinline__ int gather_rates_sel(const GridDev<Real> &G, const Sr
             const SrcSel<Real> &S = sel[s];
             if (N >= S.nst) continue;
             int i, j, k;
-            if (!(sel_lnamp(S, X, Y, Z, N, i, j, k) > lnthr)) continue;
-            if (cnt == NK) return NK + 1;
-            SrcRate<Real> t;
-            src_rate<Real>(t, G.qfac[s], G.tab[s], G.sigma0, G.dx, n, G.pcode[s] != 0, i, j, k, N, tabs);
-            if constexpr (NK <= 16) {
+            const float la = sel_lnamp(S, X, Y, Z, N, i, j, k);
+            if (!(la > lnthr)) continue;
+            if (SUM) ampsum += __expf(la);
+            m |= 1u << q;
+        }
+        mask |= (unsigned long long)m << s0;
+    }
+    return mask;
+}
+
+// The rates of selected source s at cell g, and its terms of F(x0) and F'(x0)
+// added to F and dF.
+template <typename Real>
+__device__ __forceinline__ void selected_rate(SrcRate<Real> &r, const GridDev<Real> &G, const SrcSel<Real> *sel, const Real *Ncol,
+                                              const DevTable<Real> *tabs, int X, int Y, int Z, long long g, Real n, int s,
+                                              Real x0, Real &F, Real &dF)
+{
+    const SrcSel<Real> &S = sel[s];
+    src_rate_F<Real>(r, G.qfac[s], G.tab[s], G.sigma0, G.dx, n, G.pcode[s] != 0, oct_index(X, S.v0), oct_index(Y, S.v1),
+                     oct_index(Z, S.v2), Ncol[(long long)s * G.ncell + g], tabs, x0, F, dF);
+}
+
+// Rate parameters of the selected sources, into r[0 .. NK-1] (up to four:
+// indices fixed at compile time, so r stays in registers), and their terms of
+// F(x0) and F'(x0), added to F and dF.  Returns how many there are; NK + 1 when
+// there are more than NK.
+//
+// Selecting first and forming the rates in a second loop lets the lanes of a
+// warp form the rates of different sources at a time: the loop runs as long as
+// the largest count of a lane, where rates formed as they are selected cost
+// every source that any lane selects.
+template <typename Real, int NK>
+__device__ __forceinline__ int gather_rates_sel(const GridDev<Real> &G, const SrcSel<Real> *sel, const Real *Ncol,
+                                                const DevTable<Real> *tabs, int X, int Y, int Z, long long g, Real n,
+                                                float lnthr, SrcRate<Real> *r, Real x0, Real &F, Real &dF)
+{
+    float unused = 0.0f;
+    unsigned long long mask = select_sources<Real, false>(G, sel, Ncol, X, Y, Z, g, lnthr, unused);
+    const int na = __popcll(mask);
+    if (na > NK) return NK + 1;
+    for (int cnt = 0; mask; cnt++) {
+        const int s = __ffsll(mask) - 1;
+        mask &= mask - 1;
+        SrcRate<Real> t;
+        selected_rate(t, G, sel, Ncol, tabs, X, Y, Z, g, n, s, x0, F, dF);
+        if constexpr (NK <= 4) {
 #pragma unroll
-                for (int u = 0; u < NK; u++)
-                    if (u == cnt) r[u] = t;
-            } else {
-                r[cnt] = t;                 // a local-memory array: index it directly
-            }
-            cnt++;
+            for (int u = 0; u < NK; u++)
+                if (u == cnt) r[u] = t;
+        } else {
+            r[cnt] = t;                 // a local-memory array: index it directly
         }
     }
-    return cnt;
+    return na;
 }
 
 // ln(1e-3 eps / h): the selection threshold for a step h (-inf: keep every source)
@@ -566,22 +640,27 @@ __device__ __forceinline__ bool closed_form_from_F(Real c, Real x0, Real h, Real
 // (A3's half step, A2's full step), which settles photon-free and slow cells
 // from the cache alone.  A3's full step (new columns) and the cells the cache
 // does not settle select their sources for the step and run the closed forms
-// on them; the rest go to the general pass.  The kernel walks BS-cell
-// chunks with a stride of the grid size.
-// BS: threads (and cells) per block, 128 or 256 (tuned): small blocks hold up
-// fewer cells at their barriers behind a slow one.
+// on them; the rest go to the general pass.  A block takes a run of
+// consecutive cells, as in cell_kernel.
+// BS: threads per block, 128 or 256 (tuned): small blocks hold up fewer cells
+// at their barriers behind a slow one.
+// At 512^3 cells and 16 sources the dt pass reads 8.6 GB of columns, 1.27 ms at
+// the copy rate; it and the full step take 4.8 and 5.7 ms (8.1 and 8.5 before
+// the selection was split from the rates, see gather_rates_sel, and 10 and 17
+// with the rates of tab_all formed inside the selecting loop), the half step,
+// which mostly reads the cache, 1.5 ms (2.6).  The bounds of the sources near
+// enough to matter, issued per source and cell, are what is left.
 template <typename Real, int OP, int BS>
 __global__ void __launch_bounds__(BS, (sizeof(Real) == 4 ? 1024 : 512) / BS) cell_multi_kernel(const GridDev<Real> *grids, int ngrid,
                                                          const long long *offsets, long long total,
                                                          const DevTable<Real> *tabs, unsigned *queue,
-                                                         unsigned *qcount, Real *rcache, int use_cache, int verify)
+                                                         unsigned *qcount, Real *rcache, int use_cache, int verify, int run)
 {
     __shared__ double sh[32];
     __shared__ int s_grid_lo, s_grid_hi, s_skip;
     __shared__ double s_h, s_hint;
     __shared__ float s_lnthr, s_f[4];
     constexpr bool F32 = sizeof(Real) == 4;
-    const long long nchunk = (total + BS - 1) / BS;
     if (OP == OP_RATEDT && verify) {
         // nothing to do unless some grid's first-pass minimum exceeded its hint
         if (threadIdx.x == 0) {
@@ -598,13 +677,10 @@ __global__ void __launch_bounds__(BS, (sizeof(Real) == 4 ? 1024 : 512) / BS) cel
         __syncthreads();
         if (!s_skip) return;
     }
-    for (long long chunk = blockIdx.x; chunk < nchunk; chunk += gridDim.x) {
-    const long long base = chunk * BS;
+    const long long run_lo = (long long)blockIdx.x * run, run_hi = run_lo + run < total ? run_lo + run : total;
     if (threadIdx.x == 0) {
-        long long last = base + blockDim.x - 1;
-        if (last >= total) last = total - 1;
-        s_grid_lo = find_grid(offsets, ngrid, base);
-        s_grid_hi = find_grid(offsets, ngrid, last);
+        s_grid_lo = find_grid(offsets, ngrid, run_lo);
+        s_grid_hi = find_grid(offsets, ngrid, run_hi - 1);
         if (!cells_live<Real, OP>(grids, s_grid_lo, s_grid_hi)) s_grid_hi = s_grid_lo - 1;
     }
     __syncthreads();
@@ -643,21 +719,23 @@ __global__ void __launch_bounds__(BS, (sizeof(Real) == 4 ? 1024 : 512) / BS) cel
         }
         __syncthreads();
         if (s_skip) { __syncthreads(); continue; }
-        const long long idx = base + threadIdx.x;
-        const bool mine = idx < total && idx >= offsets[gi] && (gi + 1 >= ngrid || idx < offsets[gi + 1]) &&
-                          idx - offsets[gi] >= G.cell_lo && idx - offsets[gi] < G.cell_hi;
-        const bool stepping = s_h > 0.0;
-        const bool active = mine && (OP == OP_RATEDT ? !st->done : stepping);
+        const bool live = OP == OP_RATEDT ? !st->done : s_h > 0.0;
+        const long long off = offsets[gi], gend = gi + 1 < ngrid ? offsets[gi + 1] : total;
+        // this grid's cells of the run
+        const long long clo = max(max(run_lo, off) - off, G.cell_lo), chi = min(min(run_hi, gend) - off, G.cell_hi);
+        const int cnt = live && chi > clo ? (int)(chi - clo) : 0;
+        const unsigned nx = (unsigned)G.nx, nxy = (unsigned)G.nx * (unsigned)G.ny;
         double dtmin = __longlong_as_double(0x7ff0000000000000ll);
         float dtmin_f = __int_as_float(0x7f800000);
-        float ions_f = 0.0f, rec_f = 0.0f;
+        float ions_f = 0.0f, rec_f = 0.0f, ions_e = 0.0f, rec_e = 0.0f;
         double ions = 0.0, rec = 0.0;
+        for (int o0 = 0; o0 < cnt; o0 += BS) {
         bool defer = false;
-        if (active) {
-            const long long g = idx - offsets[gi];
-            const int X = (int)(g % G.nx);
-            const int Y = (int)((g / G.nx) % G.ny);
-            const int Z = (int)(g / ((long long)G.nx * G.ny));
+        const unsigned g = (unsigned)clo + o0 + threadIdx.x;
+        if (o0 + (int)threadIdx.x < cnt) {
+            const long long idx = off + g;
+            int X, Y, Z;
+            cell_xyz(g, nx, nxy, X, Y, Z);
             const Real n = G.n ? G.n[g] : G.n_uniform;
             const Real x0 = G.x[g];
             const Real c = G.alpha * n;
@@ -670,27 +748,12 @@ __global__ void __launch_bounds__(BS, (sizeof(Real) == 4 ? 1024 : 512) / BS) cel
                 const SrcSel<Real> *sel = G.sel + (verify ? 3 : 0) * MAX_SRC;
                 float ampsum = 0.0f;
                 Real F = Real(0), dF = Real(0);
-                for (int s0 = 0; s0 < G.nsrc; s0 += 8) {
-                    Real Nb[8];
-                    load_columns8(G, G.N1, s0, g, Nb);
-#pragma unroll
-                    for (int q = 0; q < 8; q++) {
-                        const int s = s0 + q;
-                        if (s >= G.nsrc) break;
-                        const Real N = Nb[q];
-                        const SrcSel<Real> &S = sel[s];
-                        if (N >= S.nst) continue;
-                        int i, j, k;
-                        const float la = sel_lnamp(S, X, Y, Z, N, i, j, k);
-                        if (!(la > lnthr)) continue;
-                        ampsum += __expf(la);
-                        SrcRate<Real> t;
-                        src_rate<Real>(t, G.qfac[s], G.tab[s], G.sigma0, G.dx, n, G.pcode[s] != 0, i, j, k, N, tabs);
-                        Real Fs = Real(0), dFs = Real(0);
-                        src_F_term<Real>(t, tabs, x0, Fs, dFs);       // this source's term of F(x0), F'(x0)
-                        F += Fs;
-                        dF += dFs;
-                    }
+                unsigned long long mask = select_sources<Real, true>(G, sel, G.N1, X, Y, Z, g, lnthr, ampsum);
+                while (mask) {
+                    const int q = __ffsll(mask) - 1;
+                    mask &= mask - 1;
+                    SrcRate<Real> t;
+                    selected_rate(t, G, sel, G.N1, tabs, X, Y, Z, g, n, q, x0, F, dF);
                 }
                 if (rcache) {
                     rcache[idx] = F;
@@ -744,12 +807,15 @@ __global__ void __launch_bounds__(BS, (sizeof(Real) == 4 ? 1024 : 512) / BS) cel
                     SrcRate<Real> r[NACT];
                     const Real *Ncol = (OP == OP_FULL2) ? G.N2 : G.N1;
                     const SrcSel<Real> *sel = G.sel + (OP == OP_HALF ? 1 : 2) * MAX_SRC;
-                    const int na = gather_rates_sel<Real, NACT>(G, sel, Ncol, tabs, X, Y, Z, g, n, lnthr, r);
+                    // (F and F' at x0 come from the dt pass's cache, or with the rates)
+                    Real Fs = Real(0), dFs = Real(0);
+                    const int na = gather_rates_sel<Real, NACT>(G, sel, Ncol, tabs, X, Y, Z, g, n, lnthr, r, x0, Fs, dFs);
+                    if (!have_F) { F0 = Fs; dF0 = dFs; }
                     if (na <= NACT) {
                         CellODE<Real> C;
                         C.ns = na; C.c = c; C.b0 = Real(0); C.r = r; C.tabs = tabs;
                         Real f0;
-                        done = integrate_prelude<Real, NACT>(C, x0, h, G.sigma0, R, F0, dF0, f0, have_F && na > 0);
+                        done = integrate_prelude<Real, NACT>(C, x0, h, G.sigma0, R, F0, dF0, f0, na > 0);
                     }
                 }
                 if (done) {
@@ -758,12 +824,12 @@ __global__ void __launch_bounds__(BS, (sizeof(Real) == 4 ? 1024 : 512) / BS) cel
                     } else {
                         G.xout[g] = R.x;
                         if (F32) {
-                            ions_f = float(n) * (float(x0) - float(R.x));
-                            rec_f = float(n) * float(R.IR);
+                            add_two(ions_f, ions_e, float(n) * (float(x0) - float(R.x)));
+                            add_two(rec_f, rec_e, float(n) * float(R.IR));
                         } else {
                             const double nV = double(n) * st->cell_volume;
-                            ions = nV * (double(x0) - double(R.x));
-                            rec = nV * double(R.IR);
+                            ions += nV * (double(x0) - double(R.x));
+                            rec += nV * double(R.IR);
                         }
                     }
                 } else {
@@ -781,30 +847,15 @@ __global__ void __launch_bounds__(BS, (sizeof(Real) == 4 ? 1024 : 512) / BS) cel
                     atomicAdd(&st->nq[OP == OP_HALF ? 0 : 1], (unsigned)__popc(m));
                 }
                 qb = __shfl_sync(0xffffffffu, qb, leader);
-                if (defer) queue[qb + __popc(m & ((1u << lane) - 1u))] = (unsigned)idx;
+                if (defer) queue[qb + __popc(m & ((1u << lane) - 1u))] = (unsigned)(off + g);
             }
         }
+        }
         if (OP == OP_RATEDT) {
-            if (F32) {
-                for (int o = 16; o > 0; o >>= 1) dtmin_f = fminf(dtmin_f, __shfl_down_sync(0xffffffffu, dtmin_f, o));
-                if ((threadIdx.x & 31) == 0) dtmin = double(dtmin_f);
-            } else {
-                for (int o = 16; o > 0; o >>= 1) dtmin = fmin(dtmin, __shfl_down_sync(0xffffffffu, dtmin, o));
-            }
-            const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-            __syncthreads();
-            if (lane == 0) sh[wid] = dtmin;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double mn = sh[0];
-                for (int w = 1; w < (int)(blockDim.x >> 5); w++) mn = fmin(mn, sh[w]);
-                // (the read skips the atomic of a block that cannot lower the minimum)
-                const unsigned long long mb = (unsigned long long)__double_as_longlong(mn);
-                if (mn < 1e300 && mb < *(volatile unsigned long long *)&st->dt_bits) atomicMin(&st->dt_bits, mb);
-            }
+            block_dtmin<Real>(dtmin, dtmin_f, st, sh);
         } else if (OP == OP_FULL1 || OP == OP_FULL2) {
             double si = ions, sr = rec;
-            if (F32) block_sum2_f(ions_f, rec_f, st->cell_volume, si, sr, sh);
+            if (F32) block_sum2_f(ions_f + ions_e, rec_f + rec_e, st->cell_volume, si, sr, sh);
             else block_sum2(si, sr, sh);
             if (threadIdx.x == 0 && (si != 0.0 || sr != 0.0)) {
                 atomicAdd(&st->bud_step[1], si + sr);
@@ -813,8 +864,6 @@ __global__ void __launch_bounds__(BS, (sizeof(Real) == 4 ? 1024 : 512) / BS) cel
             }
         }
         __syncthreads();
-    }
-    __syncthreads();
     }
 }
 
@@ -876,16 +925,16 @@ cell_multi_general_kernel(const GridDev<Real> *grids, int ngrid, const long long
         const Real h = Real(hd);
         const float lnthr = st->lnthr[OP == OP_HALF ? 1 : 2];
         IntResult<Real> R;
-        Real F0, dF0, f0;
+        Real F0 = Real(0), dF0 = Real(0), f0;
         // the sources selected for the step (as the closed-form pass selected them),
         // in local memory; one instantiation of the integrator keeps the kernel's
         // code small (its lanes run apart through the root search and quadrature)
         SrcRate<Real> ra[MAX_SRC];
         const SrcSel<Real> *sel = G.sel + (OP == OP_HALF ? 1 : 2) * MAX_SRC;
         CellODE<Real> C;
-        C.ns = gather_rates_sel<Real, MAX_SRC>(G, sel, Ncol, tabs, X, Y, Z, g, n, lnthr, ra);
+        C.ns = gather_rates_sel<Real, MAX_SRC>(G, sel, Ncol, tabs, X, Y, Z, g, n, lnthr, ra, x0, F0, dF0);
         C.c = G.alpha * n; C.b0 = Real(0); C.r = ra; C.tabs = tabs;
-        if (!integrate_prelude<Real, MAX_SRC>(C, x0, h, G.sigma0, R, F0, dF0, f0))
+        if (!integrate_prelude<Real, MAX_SRC>(C, x0, h, G.sigma0, R, F0, dF0, f0, true))
             R = integrate_general<Real, MAX_SRC>(C, x0, h, G.sigma0, R, F0, dF0, f0, GroupEval<W>{lane, gbase, gmask});
         if (lane == 0) {
             if (OP == OP_HALF) {
@@ -949,7 +998,7 @@ cell_seq_kernel(const GridDev<Real> *grids, int ngrid, const long long *offsets,
             const Real h = Real(OP == OP_HALF ? 0.5 * st->dt : st->dt);
             SrcRate<Real> r[NSMAX];
             CellODE<Real> C;
-            Real n, x0, F0, dF0, f0;
+            Real n, x0, F0 = Real(0), dF0 = Real(0), f0;
             IntResult<Real> R;
             bool done = false;
             if (NSMAX == 1) {
@@ -965,13 +1014,13 @@ cell_seq_kernel(const GridDev<Real> *grids, int ngrid, const long long *offsets,
                 x0 = G.x[g];
                 const SrcSel<Real> *sel = G.sel + (OP == OP_HALF ? 1 : 2) * MAX_SRC;
                 C.ns = gather_rates_sel<Real, NSMAX>(G, sel, OP == OP_FULL2 ? G.N2 : G.N1, tabs, X, Y, Z, g, n,
-                                                     st->lnthr[OP == OP_HALF ? 1 : 2], r);
+                                                     st->lnthr[OP == OP_HALF ? 1 : 2], r, x0, F0, dF0);
             }
             C.c = G.alpha * n;
             C.b0 = Real(0);
             C.r = r;
             C.tabs = tabs;
-            if (NSMAX != 1) done = integrate_prelude<Real, NSMAX>(C, x0, h, G.sigma0, R, F0, dF0, f0);
+            if (NSMAX != 1) done = integrate_prelude<Real, NSMAX>(C, x0, h, G.sigma0, R, F0, dF0, f0, true);
             if (!done) R = integrate_general<Real, NSMAX>(C, x0, h, G.sigma0, R, F0, dF0, f0, SeqEval());
             if (OP == OP_HALF) {
                 const_cast<Real *>(G.xh)[g] = R.x;
@@ -1056,31 +1105,45 @@ __global__ void finalize_kernel(const GridDev<Real> *grids, int ngrid, int stage
     }
 }
 
-template <typename Real, int NSMAX, int BS>
-static cudaError_t launch_cell_ns(const GridDev<Real> *grids, int ngrid, const long long *offsets, long long total,
+// Cells of a block's run in the closed-form passes: sixteen times its threads,
+// halved while that would leave fewer than four times gen_blocks (about four
+// per SM), so that the last wave of blocks stays a small part of the pass.
+// Full step, us, at 1 / 4 / 8 / 16 / 32: 256^3 monochromatic 516 / 309 / 280 /
+// 268 / 268; 512^3 with 16 sources 7520 (4) / 6727 / 6572; a grid of 10^5 cells
+// keeps one.
+static int cell_run(long long total, int bs, int gen_blocks)
+{
+    int k = 16;
+    while (k > 1 && (total + (long long)k * bs - 1) / ((long long)k * bs) < 4LL * gen_blocks) k /= 2;
+    return k * bs;
+}
+
+template <typename Real, int BS>
+static cudaError_t launch_cell_single(const GridDev<Real> *grids, int ngrid, const long long *offsets, long long total,
                                   const DevTable<Real> *tabs, int op, unsigned *queue, unsigned *qcount,
                                   Real *qrec, Real *rcache, int use_cache, int gen_blocks, cudaStream_t s)
 {
-    const long long nb = (total + BS - 1) / BS;
+    const int run = cell_run(total, BS, gen_blocks);
+    const long long nb = (total + run - 1) / run;
     const int gbs = 256;                 // the general pass's blocks
     const bool seq = total >= (long long)seq_cells<Real>();   // its queue may be long enough for a thread per cell
     const int seq_blocks = gen_blocks * (sizeof(Real) == 4 ? 2 : 3);
     switch (op) {
-    case OP_RATEDT: cell_kernel<Real, OP_RATEDT, NSMAX, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, qrec, rcache, use_cache); break;
-    case OP_HALF: cell_kernel<Real, OP_HALF, NSMAX, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, qrec, rcache, use_cache); break;
-    case OP_FULL1: cell_kernel<Real, OP_FULL1, NSMAX, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, qrec, rcache, use_cache); break;
-    case OP_FULL2: cell_kernel<Real, OP_FULL2, NSMAX, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, qrec, rcache, use_cache); break;
+    case OP_RATEDT: cell_kernel<Real, OP_RATEDT, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, qrec, rcache, use_cache, run); break;
+    case OP_HALF: cell_kernel<Real, OP_HALF, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, qrec, rcache, use_cache, run); break;
+    case OP_FULL1: cell_kernel<Real, OP_FULL1, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, qrec, rcache, use_cache, run); break;
+    case OP_FULL2: cell_kernel<Real, OP_FULL2, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, qrec, rcache, use_cache, run); break;
     case OP_HALF | OP_GENERAL:
-        if (seq) cell_seq_kernel<Real, OP_HALF, NSMAX><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
-        cell_general_kernel<Real, OP_HALF, NSMAX><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
+        if (seq) cell_seq_kernel<Real, OP_HALF, 1><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
+        cell_general_kernel<Real, OP_HALF><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
         break;
     case OP_FULL1 | OP_GENERAL:
-        if (seq) cell_seq_kernel<Real, OP_FULL1, NSMAX><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
-        cell_general_kernel<Real, OP_FULL1, NSMAX><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
+        if (seq) cell_seq_kernel<Real, OP_FULL1, 1><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
+        cell_general_kernel<Real, OP_FULL1><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
         break;
     case OP_FULL2 | OP_GENERAL:
-        if (seq) cell_seq_kernel<Real, OP_FULL2, NSMAX><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
-        cell_general_kernel<Real, OP_FULL2, NSMAX><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
+        if (seq) cell_seq_kernel<Real, OP_FULL2, 1><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
+        cell_general_kernel<Real, OP_FULL2><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, qrec);
         break;
     default: return cudaErrorInvalidValue;
     }
@@ -1092,21 +1155,24 @@ static cudaError_t launch_cell_multi(const GridDev<Real> *grids, int ngrid, cons
                                      const DevTable<Real> *tabs, int op, unsigned *queue, unsigned *qcount,
                                      Real *rcache, int uc, int gen_blocks, cudaStream_t s)
 {
-    const long long nb = (total + BS - 1) / BS;
+    const int run = cell_run(total, BS, gen_blocks);
+    const long long nb = (total + run - 1) / run;
     const int gbs = 256;                 // the general pass's blocks
     const bool seq = total >= (long long)seq_cells<Real>();   // its queue may be long enough for a thread per cell
     const int seq_blocks = gen_blocks * (sizeof(Real) == 4 ? 2 : 3);
+    // the verifying pass: few blocks with long runs, which return unless the minimum exceeded the hint
+    const int vrun = (int)std::min<long long>(1 << 30, ((total + 8LL * gen_blocks - 1) / (8LL * gen_blocks) + BS - 1) / BS * BS);
+    const long long vnb = (total + vrun - 1) / vrun;
     switch (op) {
     case OP_RATEDT:
-        cell_multi_kernel<Real, OP_RATEDT, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 0);
+        cell_multi_kernel<Real, OP_RATEDT, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 0, run);
         break;
     case OP_RATEDT_VERIFY:
-        // the verifying pass: a few resident blocks that return unless the minimum exceeded the hint
-        cell_multi_kernel<Real, OP_RATEDT, BS><<<(unsigned)std::min<long long>(nb, 8LL * gen_blocks * (256 / BS)), BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 1);
+        cell_multi_kernel<Real, OP_RATEDT, BS><<<(unsigned)vnb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 1, vrun);
         break;
-    case OP_HALF: cell_multi_kernel<Real, OP_HALF, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 0); break;
-    case OP_FULL1: cell_multi_kernel<Real, OP_FULL1, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 0); break;
-    case OP_FULL2: cell_multi_kernel<Real, OP_FULL2, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 0); break;
+    case OP_HALF: cell_multi_kernel<Real, OP_HALF, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 0, run); break;
+    case OP_FULL1: cell_multi_kernel<Real, OP_FULL1, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 0, run); break;
+    case OP_FULL2: cell_multi_kernel<Real, OP_FULL2, BS><<<(unsigned)nb, BS, 0, s>>>(grids, ngrid, offsets, total, tabs, queue, qcount, rcache, uc, 0, run); break;
     case OP_HALF | OP_GENERAL:
         if (seq) cell_seq_kernel<Real, OP_HALF, MAX_SRC><<<seq_blocks, 128, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount, nullptr);
         cell_multi_general_kernel<Real, OP_HALF><<<gen_blocks, gbs, 0, s>>>(grids, ngrid, offsets, tabs, queue, qcount);
@@ -1137,8 +1203,8 @@ cudaError_t launch_cell(const GridDev<Real> *grids, int ngrid, const long long *
     const int uc = use_cache && rcache ? 1 : 0;
     if (nsmax <= 1)
         return cell_bs == 256
-                   ? launch_cell_ns<Real, 1, 256>(grids, ngrid, offsets, total, tabs, op, queue, qcount, qrec, rcache, uc, gen_blocks, s)
-                   : launch_cell_ns<Real, 1, 128>(grids, ngrid, offsets, total, tabs, op, queue, qcount, qrec, rcache, uc, gen_blocks, s);
+                   ? launch_cell_single<Real, 256>(grids, ngrid, offsets, total, tabs, op, queue, qcount, qrec, rcache, uc, gen_blocks, s)
+                   : launch_cell_single<Real, 128>(grids, ngrid, offsets, total, tabs, op, queue, qcount, qrec, rcache, uc, gen_blocks, s);
     return cell_bs == 256
                ? launch_cell_multi<Real, 256>(grids, ngrid, offsets, total, tabs, op, queue, qcount, rcache, uc, gen_blocks, s)
                : launch_cell_multi<Real, 128>(grids, ngrid, offsets, total, tabs, op, queue, qcount, rcache, uc, gen_blocks, s);
@@ -1152,7 +1218,7 @@ int cell_general_occupancy(int nsmax)
 {
     int nb = 0;
     cudaError_t e = nsmax <= 1
-        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, cell_general_kernel<Real, OP_FULL2, 1>, 256, 0)
+        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, cell_general_kernel<Real, OP_FULL2>, 256, 0)
         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, cell_multi_general_kernel<Real, OP_FULL2>, 256, 0);
     return (e == cudaSuccess && nb > 0) ? nb : 1;
 }

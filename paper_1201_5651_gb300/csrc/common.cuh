@@ -147,6 +147,26 @@ template <typename Real> struct DevTable {
     int K;
 };
 
+// A product that is rounded by itself, never contracted into a following sum:
+// for values that kernels with one source and with several form alike, bit for
+// bit, whatever the compiler does around them.
+OOTS_HD __forceinline__ float m_mul(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+OOTS_HD __forceinline__ double m_mul(double a, double b)
+{
+#ifdef __CUDA_ARCH__
+    return __dmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+
 template <typename Real>
 OOTS_HD __forceinline__ int tab_interval(const DevTable<Real> &T, Real lnN)
 {
@@ -221,7 +241,7 @@ OOTS_HD OOTS_NOINLINE Real tab_dlnp(const DevTable<Real> &T, Real Na, Real dN)
     if (!(piece > Real(0))) piece = rem;
     Real dt = m_log1p(piece / lo) * T.inv_dl;
     acc += dt * tab_dd(T.coef + 6 * k, t1, t1 + dt);
-    if (piece >= rem) return acc;
+    if (piece >= rem || k >= T.K - 2) return acc;   // (the last interval ends at Nhi: only rounding leaves it)
     rem -= piece;
     Real hi = Nk1 + rem;   // end column (the increment itself was used above)
     // whole intervals k+1 .. k2-1, then the partial interval k2
@@ -248,6 +268,54 @@ OOTS_HD OOTS_NOINLINE Real tab_dlnp_dN(const DevTable<Real> &T, Real N)
     int k = tab_interval(T, lnN);
     Real t = (lnN - (T.lnN_lo + Real(k) * T.dl)) * T.inv_dl;
     return tab_dpoly(T.coef + 6 * k, t) * T.inv_dl / N;
+}
+
+// ln(P(N)/Q), ln P(N + dN) - ln P(N) and d ln P / dN at N + dN in one go: the
+// three functions above with their logarithms, intervals and table reads
+// shared (one logarithm for an increment inside an interval, two for others).
+// Columns below the table and beyond it go to the functions themselves.
+template <typename Real>
+OOTS_HD __forceinline__ void tab_all(const DevTable<Real> &T, Real N, Real dN, Real &lnp, Real &dl, Real &slope)
+{
+    const Real hi = N + dN;
+    if (!(N >= T.N0 && hi <= T.Nhi && dN > Real(0))) {
+        lnp = tab_lnp(T, N);
+        dl = tab_dlnp(T, N, dN);
+        slope = tab_dlnp_dN(T, hi);
+        return;
+    }
+    const Real lnN = m_log(N);
+    int k = tab_interval(T, lnN);
+    const Real *a = T.coef + 6 * k;
+    Real t = m_mul(lnN - (T.lnN_lo + Real(k) * T.dl), T.inv_dl);
+    lnp = a[0] + t * (a[1] + t * (a[2] + t * (a[3] + t * (a[4] + t * a[5]))));
+    Real Nk1 = T.Nnode[k + 1];
+    if (Nk1 <= N && k < T.K - 2) {           // the rounding of ln N put N an interval low
+        k++;
+        a += 6;
+        Nk1 = T.Nnode[k + 1];
+        t = Real(0);
+    }
+    Real piece = m_min(Nk1 - N, dN);
+    if (!(piece > Real(0))) piece = dN;
+    const Real dt = m_mul(m_log1p(piece / N), T.inv_dl);
+    dl = m_mul(dt, tab_dd(a, t, t + dt));
+    t += dt;
+    if (piece < dN && k < T.K - 2) {         // (in the last interval only the rounding of hi gets here)
+        // whole intervals k+1 .. k2-1, then the partial interval k2
+        int k2 = tab_interval(T, m_log(hi));
+        if (k2 < k + 1) k2 = k + 1;
+        if (T.Nnode[k2] > hi && k2 > k + 1) k2--;
+        dl += T.L[k2] - T.L[k + 1];
+        const Real rem = (k2 == k + 1) ? dN - piece : hi - T.Nnode[k2];
+        a = T.coef + 6 * k2;
+        t = Real(0);
+        if (rem > Real(0)) {
+            t = m_mul(m_log1p(rem / T.Nnode[k2]), T.inv_dl);
+            dl += m_mul(t, tab_dd(a, Real(0), t));
+        }
+    }
+    slope = m_mul(tab_dpoly(a, t), T.inv_dl) / hi;
 }
 
 // ---------------------------------------------------------------------------
@@ -289,6 +357,28 @@ OOTS_HD __forceinline__ void src_rate(SrcRate<Real> &r, Real qfac, int tab, Real
         r.A = qfac / den;
         r.b = n * dx * sf;
         if (with_p) r.p = m_exp(tab_lnp(tabs[tab], N));
+    }
+}
+
+// src_rate and the source's term of F(x) and F'(x), added to F and dF.
+template <typename Real>
+OOTS_HD __forceinline__ void src_rate_F(SrcRate<Real> &r, Real qfac, int tab, Real sigma0, Real dx, Real n, bool plane,
+                                        int i, int j, int k, Real N, const DevTable<Real> *tabs, Real x, Real &F, Real &dF)
+{
+    src_rate<Real>(r, qfac, tab, sigma0, dx, n, plane, i, j, k, N, tabs, false);
+    if (tab < 0) {
+        if (!(r.A > Real(0))) return;
+        const Real e = m_expm1(-m_mul(r.b, x));
+        F -= m_mul(r.A, e);
+        dF += m_mul(m_mul(r.A, r.b), Real(1) + e);
+    } else {
+        Real lnp, dl, slope;
+        tab_all(tabs[tab], N, m_mul(r.b, x), lnp, dl, slope);
+        r.p = m_exp(lnp);
+        if (!(r.A > Real(0))) return;
+        F -= m_mul(m_mul(r.A, r.p), m_expm1(dl));
+        const Real px = m_mul(r.p, m_exp(dl));
+        if (px > Real(0)) dF -= m_mul(m_mul(m_mul(r.A, px), r.b), slope);
     }
 }
 
