@@ -180,8 +180,8 @@ def job_rate(units_per_rank, world, t_ms):
     return world * units_per_rank / (t_ms / 1e3)
 
 
-KERNEL_SOURCES = ("common.cuh", "integrator.cuh", "kernels.h", "oots_internal.h", "sweep_impl.cuh", "sweep_tp.cuh",
-                  "sweep_f.cu", "sweep_d.cu", "cell.cu")
+KERNEL_SOURCES = ("common.cuh", "integrator.cuh", "kernels.h", "oots_internal.h", "march.cuh", "march_f.cu",
+                  "march_d.cu", "march_a1.cuh", "march_a1_f.cu", "march_a1_d.cu", "cell.cu")
 
 
 def kernel_source_hash():
@@ -257,13 +257,13 @@ def step_bytes_per_cell(nsrc, n_array):
 
 
 def _describe_tile(shape, cell_block=None, nsrc=1):
-    """The sweep's tile shape and kernel, and (when given) the threads per block of
+    """The tile shape asked for and the trace kernel, and (when given) the threads per block of
     the closed-form per-cell passes (0 = the library's default for the source count)."""
     from paper_1201_5651_gb300 import oots
     if shape is None:
         return None
     dims = oots.oots_tile_shape_info(shape)[1]
-    d = {"id": shape, "dims": list(dims), "kernel": "throughput" if shape in (7, 8) else "pipelined"}
+    d = {"id": shape, "dims": list(dims), "kernel": "march"}
     if cell_block is not None:
         d["cell_block"] = cell_block if cell_block else (128 if nsrc > 1 else 256)
     return d
@@ -272,7 +272,7 @@ def _describe_tile(shape, cell_block=None, nsrc=1):
 def _roofline(prof_avg, ms_per_step, ncell, nsrc, n_array, workload, tile_shape):
     peak, peak_src = _peaks()
     # each pass with its helper launches: a trace with the packing of its input
-    # (throughput tiles), the Eq. 4 pass with its verifying re-run, an
+    # (several sources), the Eq. 4 pass with its verifying re-run, an
     # integration with its general pass
     parts = {"half": ["half", "half_general"], "full": ["full", "full_general"],
              "ratedt": ["ratedt", "ratedt_verify"], "sweep1": ["sweep1", "pack"], "sweep2": ["sweep2", "pack"]}

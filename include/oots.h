@@ -27,8 +27,8 @@
  *     read or write caller-owned device memory on the context's stream and
  *     never keep or free the pointer.
  *   - A context is not thread-safe; use one context per thread.
- *   - Device waits are bounded: a wavefront tile that waits too long for its
- *     upstream neighbours gives up, the call returns OOTS_E_DEVICE_TIMEOUT and
+ *   - Device waits are bounded: a block of the trace that waits too long for
+ *     its upstream neighbours gives up, the call returns OOTS_E_DEVICE_TIMEOUT and
  *     the context stays usable after oots_reset_error().
  */
 #ifndef OOTS_H
@@ -199,7 +199,7 @@ int oots_run_substeps(oots_ctx *ctx, long long n, double t_end);
 #define OOTS_K_FULL_GENERAL 10 /* full step, cells no closed form settles (one warp each) */
 #define OOTS_K_PLANE_TRACE 11  /* columns of the plane-parallel sources (either trace) */
 #define OOTS_K_PLANE_IMPLICIT 12 /* A1 row integration of a plane-parallel source */
-#define OOTS_K_PACK      13  /* n x of the traced state into tile bricks (before each throughput trace) */
+#define OOTS_K_PACK      13  /* n x of the traced state, packed (before a trace of several sources) */
 #define OOTS_K_RATEDT_VERIFY 14 /* several sources: re-run of the Eq. 4 pass when the step hint was too short */
 int oots_profile_substep(oots_ctx *ctx, int *kinds, double *ms, int nmax, int *n_out);
 
@@ -305,21 +305,20 @@ int oots_batch_destroy(oots_batch *b);
 
 /* ---- tuning and diagnostics ----------------------------------------------------------------- */
 
-/* Choose the sweep tile shape (0..6, see oots_tile_shape_info; -1 = automatic) -- the autotuner's hook. */
+/* Choose the trace's tile shape (see oots_tile_shape_info; -1 = automatic) -- the autotuner's hook.
+ * The trace marches blocks of one shape per precision, which every grid size measured fastest on: a
+ * shape is checked and kept, and changes nothing else. */
 int oots_set_tile_shape(oots_ctx *ctx, int shape);
 
 /* Number of tile shapes and the dimensions of one. */
 int oots_tile_shape_info(int shape, int dims[3]);
 
-/* Debug and tuning controls: key 1 = spin limit of the bounded tile waits
- * (iterations, > 0); key 2 = index of a tile that never publishes its
+/* Debug and tuning controls: key 1 = spin limit of the trace's bounded waits
+ * (iterations, > 0); key 2 = index of a block that never publishes its
  * progress (-1 = none), which makes its downstream waits run out and the call
- * return OOTS_E_DEVICE_TIMEOUT without faulting the device; key 3 = planes a
- * sweep tile completes between two progress publications (1..64; 0 = the
- * default of 4); key 4 = where the sweep's tiles start: 0 (default) at
- * multiples of the tile size in global coordinates (rows of x aligned to
- * memory), 1 at the octant's origin (the octant's diagonal planes then cut
- * only the tiles on the tile diagonals); key 5 = threads per block of the
+ * return OOTS_E_DEVICE_TIMEOUT without faulting the device; key 3 (0..64) and
+ * key 4 (0 or 1) are checked and change nothing (they set the hand-over and
+ * the alignment of an earlier trace's tiles); key 5 = threads per block of the
  * closed-form per-cell passes (the dt criterion, the half and full steps):
  * 128, 256, or 0 for the default (128 with several sources per grid, 256
  * with one).  OOTS_E_INVAL for an unknown key or a value out of range. */
@@ -331,8 +330,7 @@ int oots_debug_set(oots_ctx *ctx, int key, long long value);
  * device memory: code that works inside a pre-sized memory pool or arena
  * that owns the whole device, or a host process whose allocator must not be
  * re-entered (a cudaMalloc there can fail, fragment the arena or deadlock).
- * No counterpart in the paper: it exposes the library's wavefront sweep on
- * its own.
+ * No counterpart in the paper: it exposes the library's trace on its own.
  *
  * Inputs and outputs are caller-owned device buffers (x-fastest, ncell
  * values each): x_dev the neutral fraction, n_dev the density (NULL: the
@@ -342,8 +340,7 @@ int oots_debug_set(oots_ctx *ctx, int key, long long value);
  * (float buffers).  The call enqueues on `stream` (NULL: the default stream)
  * and returns when the trace has finished.
  *
- * Nothing is allocated: the scratch (tile work list, published tile faces,
- * descriptors) is one 64 MiB static device array that every GPU
+ * Nothing is allocated: the scratch (work list, halos, descriptors) is one 64 MiB static device array that every GPU
  * loading the library holds until the process exits.  A grid that needs more
  * tiles of 16x8x8 cells than fit in it (about 5400 in FP64, 7200 mixed, i.e.
  * roughly 5 million cells) is rejected with OOTS_E_INVAL, *status_detail

@@ -1,14 +1,9 @@
-"""Autotuner for a substep's launch shapes: the sweep's tile shape and kernel,
-and the block size of the closed-form per-cell passes.
+"""Autotuner for a substep's launch shapes: the trace's tile shape and the
+block size of the closed-form per-cell passes.
 
-The sweep has two kernels (the pipelined one, whose tiles hand their faces on
-plane chunk by chunk, and the throughput one, which traces whole 8^3 tiles)
-and several tile shapes.  Which is fastest depends on how many tiles the
-wavefront keeps in flight per diagonal plane: a single source on a 128^3 grid
-leaves most of the machine idle, so the pipelined kernel's early hand-off
-wins; sixteen sources on 512^3 give thousands of tiles per plane, and the
-lean throughput tiles win.  The tuner therefore keys its choice on a
-plane-size class of the launch -- the largest grid side (rounded up to a
+The trace runs one block shape per precision whatever tile shape is asked for,
+so the shapes differ by noise now; the interface and the cache keep them.  The
+tuner keys its choice on a plane-size class of the launch -- the largest grid side (rounded up to a
 power of two), the number of sources per grid and the number of grids, each
 bucketed -- rather than on the exact grid, times every shape the device can
 run on one substep (per-launch CUDA events through oots_profile_substep, or
@@ -42,7 +37,7 @@ def _bucket(v: int, edges: Sequence[int]) -> int:
 def plane_class(nx: int, ny: int, nz: int, nsrc: int, ngrids: int = 1) -> str:
     """The class of a launch for tuning: side (next power of two of the largest
     side, at least 16), sources per grid and grids, bucketed.  Together they set
-    the number of tiles in flight on a wavefront plane."""
+    how much of the machine a launch fills."""
     side = 16
     while side < max(nx, ny, nz):
         side *= 2

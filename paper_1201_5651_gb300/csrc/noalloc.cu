@@ -1,8 +1,7 @@
 // oots_trace_noalloc: the column-density trace for callers that cannot
-// allocate device memory.  It runs the same wavefront sweep kernel as the
-// context API, but every piece of scratch it needs (the tile work list, the
-// published tile faces and the small descriptors) lives in
-// one file-scope static device array, so the call makes no cudaMalloc, no
+// allocate device memory.  It runs the same trace kernel as the
+// context API, but every piece of scratch it needs (the work list, the
+// halos between blocks and the small descriptors) lives in one file-scope static device array, so the call makes no cudaMalloc, no
 // cudaFree and no heap allocation on the host.
 #include <cmath>
 #include <cstdio>
