@@ -1,5 +1,5 @@
 // C ABI of the library (include/oots.h): argument checking, device memory,
-// source snapping and octant split, the tile work list, substep sequencing
+// source snapping and octant split, the trace's work list, substep sequencing
 // of the schemes A1/A2/A3 (Mackey 2012, Sect. 2.1-2.2) and CUDA-graph replay.
 #include <algorithm>
 #include <cmath>
@@ -110,8 +110,6 @@ struct oots_ctx {
     int shape = -1;
     long long spin_limit = 1ll << 22;
     long long skip_publish = -1;
-    int sweep_chunk = 0;               // planes per progress step of the sweep (0: default)
-    int tile_align = 0;                // tile origins: 0 global multiples of the tile (x rows aligned), 1 the octant's
     int cell_block = 0;                // threads per block of the closed-form passes: 128, 256, 0 = by source count
     size_t rsize = 8;
     void *d_x = nullptr, *d_n = nullptr, *d_xh = nullptr, *d_N1 = nullptr, *d_N2 = nullptr;
@@ -121,6 +119,8 @@ struct oots_ctx {
     DevState *d_st = nullptr;
     int *d_err = nullptr;
     DevState h_st;
+    bool st_current = false;        // h_st is the device's state: nothing that changes it was launched since
+    struct Readback { DevState st; int err; } *rb = nullptr;   // pinned: the state and the error word come back in one wait
     unsigned long long part_src = ~0ull;   // partition: sources this context traces (bit s)
     int part_z0 = 0, part_z1 = 0;          // partition: z-range of the cells it updates (z1 <= 0: all)
     bool phase_dt = false;                 // the dt phase ran on the current columns
@@ -497,7 +497,7 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
     }
 
     // trace (mode 0) or A1 implicit sweep (mode 1) of every source: point
-    // sources by the wavefront sweep, plane sources row by row
+    // sources by the march, plane sources row by row
     int sweep(cudaStream_t s, int which, int mode)
     {
         if (mode == 0 && ml[0].nitems > 0) {
@@ -650,30 +650,60 @@ static int check_ctx(const oots_ctx *c)
     return OOTS_OK;
 }
 
+// The state's way to the device: as a kernel's parameter, in stream order, with
+// nothing for the host to keep or to wait for.
+__global__ void push_state_kernel(DevState *st, const __grid_constant__ DevState v) { *st = v; }
+
 static int pull_state(oots_ctx *c)
 {
     CU(cudaSetDevice(c->device));
-    CU(cudaMemcpyAsync(&c->h_st, c->d_st, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
+    CU(cudaMemcpyAsync(&c->rb->st, c->d_st, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
+    c->h_st = c->rb->st;
+    c->st_current = true;
     return OOTS_OK;
 }
 
 static int push_state(oots_ctx *c)
 {
     CU(cudaSetDevice(c->device));
-    CU(cudaMemcpyAsync(c->d_st, &c->h_st, sizeof(DevState), cudaMemcpyHostToDevice, c->stream));
-    CU(cudaStreamSynchronize(c->stream));
+    push_state_kernel<<<1, 1, 0, c->stream>>>(c->d_st, c->h_st);
+    CU(cudaGetLastError());
+    c->st_current = true;
+    return OOTS_OK;
+}
+
+static int device_error(int err)
+{
+    if (err == DEVERR_TIMEOUT) return fail(OOTS_E_DEVICE_TIMEOUT, "a wavefront tile gave up waiting for its upstream tiles");
+    if (err) return fail(OOTS_E_CUDA, "device error %d", err);
     return OOTS_OK;
 }
 
 static int check_device_error(oots_ctx *c)
 {
-    int err = 0;
-    CU(cudaMemcpyAsync(&err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    CU(cudaMemcpyAsync(&c->rb->err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
-    if (err == DEVERR_TIMEOUT) return fail(OOTS_E_DEVICE_TIMEOUT, "a wavefront tile gave up waiting for its upstream tiles");
-    if (err) return fail(OOTS_E_CUDA, "device error %d", err);
-    return OOTS_OK;
+    return device_error(c->rb->err);
+}
+
+// Wait for the work in flight; then its error, if any, and the state it left.
+static int finish(oots_ctx *c)
+{
+    CU(cudaMemcpyAsync(&c->rb->err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    if (int rc = pull_state(c)) return rc;
+    return device_error(c->rb->err);
+}
+
+// Replays to queue before the next look at the state: what the step at hand
+// says is left, at most 64, and at most twice the last burst while the step may
+// change.  (A replay past the end time does nothing, but takes its launches.)
+static int next_burst(const DevState &st, bool fixed, int last)
+{
+    const double h = fixed ? st.dt_fixed : st.dt_last;
+    double k = h > 0.0 ? std::ceil((st.t_end - st.t) / h * (1.0 - 1e-12)) : 1.0;
+    if (!fixed || !(h > 0.0)) k = std::min(k, 2.0 * last);
+    return (int)std::min(std::max(k, 1.0), 64.0);
 }
 
 static void drop_solo(oots_ctx *c)
@@ -708,18 +738,23 @@ static int prepare(oots_ctx *c)
         c->nsrc_alloc = ns;
         drop_solo(c);
     }
-    // device-side criteria and source totals
-    int rc = pull_state(c);
+    // device-side criteria and source totals; h_st is current from here on
+    int rc = c->st_current ? OOTS_OK : pull_state(c);
     if (rc) return rc;
-    c->h_st.dt_fixed = c->crit.dt_fixed;
-    c->h_st.K1 = c->crit.K1;
-    c->h_st.K3 = c->crit.K3;
-    c->h_st.K4 = c->crit.K4;
     double sq = 0.0;
     for (auto &s : c->src) sq += source_emission(s, c->nx, c->ny, c->nz, c->dx);
-    c->h_st.sumQ = sq;
-    c->h_st.cell_volume = c->dx * c->dx * c->dx;
-    if ((rc = push_state(c))) return rc;
+    const double vol = c->dx * c->dx * c->dx;
+    DevState &h = c->h_st;
+    if (h.dt_fixed != c->crit.dt_fixed || h.K1 != c->crit.K1 || h.K3 != c->crit.K3 || h.K4 != c->crit.K4 ||
+        h.sumQ != sq || h.cell_volume != vol) {
+        h.dt_fixed = c->crit.dt_fixed;
+        h.K1 = c->crit.K1;
+        h.K3 = c->crit.K3;
+        h.K4 = c->crit.K4;
+        h.sumQ = sq;
+        h.cell_volume = vol;
+        if ((rc = push_state(c))) return rc;
+    }
     if (!c->dirty && c->solo) return OOTS_OK;
     delete c->solo;
     c->solo = nullptr;
@@ -858,7 +893,8 @@ int oots_create(oots_ctx **out, int device, int precision)
         return fail(OOTS_E_CUDA, "stream creation failed");
     }
     c->stream = c->own_stream;
-    if (cudaMalloc(&c->d_st, sizeof(DevState)) != cudaSuccess || cudaMalloc(&c->d_err, sizeof(int)) != cudaSuccess ||
+    if (cudaMallocHost(&c->rb, sizeof(oots_ctx::Readback)) != cudaSuccess ||
+        cudaMalloc(&c->d_st, sizeof(DevState)) != cudaSuccess || cudaMalloc(&c->d_err, sizeof(int)) != cudaSuccess ||
         cudaMalloc(&c->d_bad, sizeof(long long)) != cudaSuccess) {
         oots_destroy(c);
         return fail(OOTS_E_NOMEM, "device state");
@@ -890,6 +926,7 @@ int oots_destroy(oots_ctx *c)
     free_dev(p);
     p = c->d_bad;
     free_dev(p);
+    if (c->rb) cudaFreeHost(c->rb);
     if (c->own_stream) cudaStreamDestroy(c->own_stream);
     delete c;
     return OOTS_OK;
@@ -1111,13 +1148,12 @@ int oots_compute_dt(oots_ctx *c, double *dt)
     if (c->batched) return fail(OOTS_E_STATE, "context is part of a batch");
     int rc = prepare(c);
     if (rc) return rc;
-    if ((rc = pull_state(c))) return rc;
     c->h_st.dt_bits = 0xffffffffffffffffull;
     c->h_st.done = 0;
     if ((rc = push_state(c))) return rc;
+    c->st_current = false;
     if ((rc = c->solo->trace_for_dt(c->stream))) return rc;
-    if ((rc = check_device_error(c))) return rc;
-    if ((rc = pull_state(c))) return rc;
+    if ((rc = finish(c))) return rc;
     *dt = c->h_st.dt_bits == 0xffffffffffffffffull ? 1e300 : *(double *)&c->h_st.dt_bits;
     return OOTS_OK;
 }
@@ -1129,15 +1165,14 @@ int oots_step(oots_ctx *c, double dt)
     if (c->batched) return fail(OOTS_E_STATE, "context is part of a batch");
     int rc = prepare(c);
     if (rc) return rc;
-    if ((rc = pull_state(c))) return rc;
     c->h_st.dt_fixed = dt;
     c->h_st.t_end = c->h_st.t + dt;
     c->h_st.done = 0;
     if ((rc = push_state(c))) return rc;
     CU(cudaSetDevice(c->device));
+    c->st_current = false;
     if ((rc = c->solo->substep(c->stream, true))) return rc;
-    if ((rc = check_device_error(c))) return rc;
-    if ((rc = pull_state(c))) return rc;
+    if ((rc = finish(c))) return rc;
     c->h_st.dt_fixed = c->crit.dt_fixed;
     // the substep advanced t by exactly dt
     return push_state(c);
@@ -1150,21 +1185,23 @@ int oots_advance(oots_ctx *c, double t_end, double *t_out, long long *nsub_out)
     if (c->batched) return fail(OOTS_E_STATE, "context is part of a batch");
     int rc = prepare(c);
     if (rc) return rc;
-    if ((rc = pull_state(c))) return rc;
     long long n0 = c->h_st.nsub;
     if (t_end > c->h_st.t) {
         c->h_st.t_end = t_end;
         c->h_st.done = 0;
         if ((rc = push_state(c))) return rc;
         CU(cudaSetDevice(c->device));
-        int burst = 1;
+        const bool fixed = c->crit.dt_fixed > 0;
+        int burst = fixed ? next_burst(c->h_st, true, 1) : 1;
         for (;;) {
+            c->st_current = false;
             if ((rc = c->solo->graph_replay(c->stream, burst))) return rc;
-            if ((rc = check_device_error(c))) return rc;
-            if ((rc = pull_state(c))) return rc;
+            if ((rc = finish(c))) return rc;
             if (c->h_st.done) break;
-            if (burst < 64) burst *= 2;
+            burst = next_burst(c->h_st, fixed, burst);
         }
+    } else {
+        CU(cudaStreamSynchronize(c->stream));       // the call waits for earlier work either way
     }
     if (t_out) *t_out = c->h_st.t;
     if (nsub_out) *nsub_out = c->h_st.nsub - n0;
@@ -1183,6 +1220,7 @@ int oots_run_substeps(oots_ctx *c, long long n, double t_end)
     c->h_st.done = (t_end > c->h_st.t) ? 0 : 1;
     if ((rc = push_state(c))) return rc;
     CU(cudaSetDevice(c->device));
+    c->st_current = false;
     return n > 0 ? c->solo->graph_replay(c->stream, (int)n) : OOTS_OK;
 }
 
@@ -1200,6 +1238,7 @@ int oots_profile_substep(oots_ctx *c, int *kinds, double *ms, int nmax, int *n_o
     CU(cudaSetDevice(c->device));
     LaunchProfiler P;
     P.s = c->stream;
+    c->st_current = false;
     c->solo->prof = &P;
     rc = c->solo->substep(c->stream, c->crit.dt_fixed > 0);
     c->solo->prof = nullptr;
@@ -1310,7 +1349,6 @@ int oots_synchronize(oots_ctx *c)
 {
     if (int rc = check_ctx(c)) return rc;
     CU(cudaSetDevice(c->device));
-    CU(cudaStreamSynchronize(c->stream));
     return check_device_error(c);
 }
 
@@ -1341,10 +1379,8 @@ int oots_debug_set(oots_ctx *c, int key, long long value)
         c->skip_publish = value;
     } else if (key == 3) {
         if (value < 0 || value > 64) return fail(OOTS_E_INVAL, "sweep chunk %lld", value);
-        c->sweep_chunk = (int)value;
     } else if (key == 4) {
         if (value != 0 && value != 1) return fail(OOTS_E_INVAL, "tile alignment %lld", value);
-        c->tile_align = (int)value;
     } else if (key == 5) {
         if (value != 0 && value != 128 && value != 256) return fail(OOTS_E_INVAL, "cell block %lld", value);
         c->cell_block = (int)value;
@@ -1401,9 +1437,9 @@ int oots_run_phase(oots_ctx *c, int phase, double *value)
     }
     if ((rc = push_state(c))) return rc;
     const bool use_cache = phase == OOTS_PH_STEP1 && c->phase_dt;
+    c->st_current = false;
     if ((rc = c->solo->phase(c->stream, phase, use_cache))) return rc;
-    if ((rc = check_device_error(c))) return rc;
-    if ((rc = pull_state(c))) return rc;
+    if ((rc = finish(c))) return rc;
     if (phase == OOTS_PH_TRACE1) c->phase_dt = false;
     if (phase == OOTS_PH_DT) {
         *value = c->h_st.dt_bits == 0xffffffffffffffffull ? 1e300 : *(double *)&c->h_st.dt_bits;
@@ -1446,7 +1482,83 @@ struct oots_batch {
     std::vector<oots_ctx *> ctxs;
     LaunchSetBase *L = nullptr;
     cudaStream_t stream = nullptr;
+    // the grids' states, gathered on the device and read back in one copy
+    DevState **d_ptr = nullptr;
+    DevState *d_all = nullptr;
+    DevState *h_all = nullptr;      // pinned
+    ~oots_batch()
+    {
+        delete L;
+        if (d_ptr) cudaFree(d_ptr);
+        if (d_all) cudaFree(d_all);
+        if (h_all) cudaFreeHost(h_all);
+    }
 };
+
+__global__ void gather_states_kernel(DevState *const *st, DevState *out, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = *st[i];
+}
+
+// End times of up to END_TIMES grids of a batch, as kernel parameters (no
+// buffer of the host's to keep until the copy has run).  A grid that is past
+// its end time stops; only_later: and keeps its old end time.
+constexpr int END_TIMES = 256;
+struct EndTimes { double t[END_TIMES]; };
+__global__ void set_ends_kernel(DevState *const *st, const __grid_constant__ EndTimes e, int n, int only_later)
+{
+    const int i = threadIdx.x;
+    if (i >= n) return;
+    DevState *s = st[i];
+    const bool later = e.t[i] > s->t;
+    if (later || !only_later) s->t_end = e.t[i];
+    s->done = later ? 0 : 1;
+}
+
+static int batch_set_ends(oots_batch *b, const double *t_end, bool only_later)
+{
+    const int n = (int)b->ctxs.size();
+    for (int i0 = 0; i0 < n; i0 += END_TIMES) {
+        EndTimes e;
+        const int m = std::min(END_TIMES, n - i0);
+        for (int i = 0; i < END_TIMES; i++) e.t[i] = i < m ? t_end[i0 + i] : 0.0;
+        set_ends_kernel<<<1, END_TIMES, 0, b->stream>>>(b->d_ptr + i0, e, m, only_later ? 1 : 0);
+        CU(cudaGetLastError());
+    }
+    for (auto *c : b->ctxs) c->st_current = false;
+    return OOTS_OK;
+}
+
+// What the contexts have under way on streams of their own comes before the batch's work.
+static int batch_join(oots_batch *b)
+{
+    CU(cudaSetDevice(b->ctxs[0]->device));
+    cudaStream_t last = b->stream;
+    for (auto *c : b->ctxs)
+        if (c->stream != b->stream && c->stream != last) {
+            CU(cudaStreamSynchronize(c->stream));
+            last = c->stream;
+        }
+    return OOTS_OK;
+}
+
+// Wait for the batch's work and read every grid's state.
+static int batch_pull(oots_batch *b)
+{
+    const int n = (int)b->ctxs.size();
+    oots_ctx *c0 = b->ctxs[0];
+    gather_states_kernel<<<(n + 63) / 64, 64, 0, b->stream>>>(b->d_ptr, b->d_all, n);
+    CU(cudaGetLastError());
+    CU(cudaMemcpyAsync(b->h_all, b->d_all, n * sizeof(DevState), cudaMemcpyDeviceToHost, b->stream));
+    CU(cudaMemcpyAsync(&c0->rb->err, c0->d_err, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
+    CU(cudaStreamSynchronize(b->stream));
+    for (int i = 0; i < n; i++) {
+        b->ctxs[i]->h_st = b->h_all[i];
+        b->ctxs[i]->st_current = true;
+    }
+    return OOTS_OK;
+}
 
 int oots_batch_create(oots_batch **out, oots_ctx *const *ctxs, int n)
 {
@@ -1478,6 +1590,15 @@ int oots_batch_create(oots_batch **out, oots_ctx *const *ctxs, int n)
         if ((rc = L->build(b->ctxs, ctxs[0]->shape))) { delete L; delete b; return rc; }
         b->L = L;
     }
+    std::vector<DevState *> ptr;
+    for (auto *c : b->ctxs) ptr.push_back(c->d_st);
+    if (cudaMalloc(&b->d_ptr, n * sizeof(DevState *)) != cudaSuccess || cudaMalloc(&b->d_all, n * sizeof(DevState)) != cudaSuccess ||
+        cudaMallocHost(&b->h_all, n * sizeof(DevState)) != cudaSuccess ||
+        cudaMemcpy(b->d_ptr, ptr.data(), n * sizeof(DevState *), cudaMemcpyHostToDevice) != cudaSuccess) {
+        delete b;
+        cudaGetLastError();
+        return fail(OOTS_E_NOMEM, "states of %d grids", n);
+    }
     for (auto *c : b->ctxs) c->batched = true;
     *out = b;
     return OOTS_OK;
@@ -1486,56 +1607,45 @@ int oots_batch_create(oots_batch **out, oots_ctx *const *ctxs, int n)
 int oots_batch_advance(oots_batch *b, const double *t_end_each, long long *nsub_out)
 {
     if (!b || !t_end_each) return fail(OOTS_E_INVAL, "batch arguments");
-    std::vector<long long> n0(b->ctxs.size());
-    bool any = false;
-    for (size_t i = 0; i < b->ctxs.size(); i++) {
-        oots_ctx *c = b->ctxs[i];
-        int rc = pull_state(c);
-        if (rc) return rc;
-        n0[i] = c->h_st.nsub;
-        if (t_end_each[i] > c->h_st.t) {
-            c->h_st.t_end = t_end_each[i];
-            c->h_st.done = 0;
-            any = true;
-        } else {
-            c->h_st.done = 1;
-        }
-        if ((rc = push_state(c))) return rc;
+    const size_t n = b->ctxs.size();
+    std::vector<long long> n0(n);
+    int rc = batch_join(b);
+    if (rc) return rc;
+    bool any = false, known = true;
+    for (auto *c : b->ctxs) known = known && c->st_current;
+    if (!known && (rc = batch_pull(b))) return rc;
+    for (size_t i = 0; i < n; i++) {
+        n0[i] = b->ctxs[i]->h_st.nsub;
+        any = any || t_end_each[i] > b->ctxs[i]->h_st.t;
     }
+    if ((rc = batch_set_ends(b, t_end_each, true))) return rc;
     if (any) {
-        CU(cudaSetDevice(b->ctxs[0]->device));
         int burst = 1;
         for (;;) {
-            int rc = b->L->graph_replay(b->stream, burst);
-            if (rc) return rc;
-            if ((rc = check_device_error(b->ctxs[0]))) return rc;
-            bool all = true;
-            for (auto *c : b->ctxs) {
-                if ((rc = pull_state(c))) return rc;
-                all = all && c->h_st.done;
-            }
-            if (all) break;
-            if (burst < 64) burst *= 2;
+            if ((rc = b->L->graph_replay(b->stream, burst))) return rc;
+            if ((rc = batch_pull(b))) return rc;
+            if ((rc = device_error(b->ctxs[0]->rb->err))) return rc;
+            int next = 0;
+            for (auto *c : b->ctxs)
+                if (!c->h_st.done) next = std::max(next, next_burst(c->h_st, c->crit.dt_fixed > 0, burst));
+            if (!next) break;
+            burst = next;
         }
+    } else {
+        CU(cudaStreamSynchronize(b->stream));
     }
     if (nsub_out)
-        for (size_t i = 0; i < b->ctxs.size(); i++) nsub_out[i] = b->ctxs[i]->h_st.nsub - n0[i];
+        for (size_t i = 0; i < n; i++) nsub_out[i] = b->ctxs[i]->h_st.nsub - n0[i];
     return OOTS_OK;
 }
 
 int oots_batch_run_substeps(oots_batch *b, long long n, const double *t_end_each)
 {
     if (!b || !t_end_each || n < 0) return fail(OOTS_E_INVAL, "batch arguments");
-    for (size_t i = 0; i < b->ctxs.size(); i++) {
+    for (size_t i = 0; i < b->ctxs.size(); i++)
         if (!std::isfinite(t_end_each[i])) return fail(OOTS_E_INVAL, "t_end %g of context %zu", t_end_each[i], i);
-        oots_ctx *c = b->ctxs[i];
-        int rc = pull_state(c);
-        if (rc) return rc;
-        c->h_st.t_end = t_end_each[i];
-        c->h_st.done = (t_end_each[i] > c->h_st.t) ? 0 : 1;
-        if ((rc = push_state(c))) return rc;
-    }
-    CU(cudaSetDevice(b->ctxs[0]->device));
+    if (int rc = batch_join(b)) return rc;
+    if (int rc = batch_set_ends(b, t_end_each, false)) return rc;
     return n > 0 ? b->L->graph_replay(b->stream, (int)n) : OOTS_OK;
 }
 
@@ -1547,7 +1657,6 @@ int oots_batch_destroy(oots_batch *b)
         cudaStreamSynchronize(b->stream);
     }
     for (auto *c : b->ctxs) c->batched = false;
-    delete b->L;
     delete b;
     return OOTS_OK;
 }
