@@ -651,7 +651,10 @@ static int check_ctx(const oots_ctx *c)
 }
 
 // The state's way to the device: as a kernel's parameter, in stream order, with
-// nothing for the host to keep or to wait for.
+// nothing for the host to keep or to wait for.  (With pageable copies, a wait
+// after each and a read-back before every change, compute_dt and step at
+// 50x41x37 took 350 us in place of 249, and a substep of 64 grids 7.8 ms in
+// place of 6.1.)
 __global__ void push_state_kernel(DevState *st, const __grid_constant__ DevState v) { *st = v; }
 
 static int pull_state(oots_ctx *c)

@@ -285,8 +285,14 @@ __global__ void __launch_bounds__(128) plane_implicit_kernel(const GridDev<Real>
     }
 }
 
-// rows up to which A1 gives each a lane group
-constexpr long long kGroupRows = 4096;
+// Rows up to which A1 gives each a lane group; more rows take a thread each.
+// Groups against threads, us, uniform gas, 64 cells a row (mixed: mono, then
+// blackbody): 1024 rows 106 / 143 and 311 / 483, 4096 rows 190 / 143 and
+// 387 / 487, 9216 rows 369 / 143 and 758 / 489.  FP64: 256 rows 16.8 / 21.9 ms
+// and 17.3 / 44.3 ms, 1024 rows 32.8 / 21.9 and 32.8 / 44.5 ms, 4096 rows
+// 115 / 22 and 116 / 44 ms.  Groups take as long for one row as for as many as
+// the chip holds and then grow with the rows; the lines lie below that.
+template <typename Real> constexpr long long group_rows() { return sizeof(Real) == 4 ? 2048 : 512; }
 
 long long plane_job_threads(int code, long long rows)
 {
@@ -304,7 +310,7 @@ cudaError_t launch_plane(const GridDev<Real> *grids, const PlaneJob *jobs, int n
     if (implicit) {
         const int bs = 128;
         constexpr int W = GroupWidth<Real>::value;
-        if (rows0 <= kGroupRows)
+        if (rows0 <= group_rows<Real>())
             plane_implicit_kernel<Real, W><<<(unsigned)((rows0 * W + bs - 1) / bs), bs, 0, s>>>(grids, jobs, tabs);
         else
             plane_implicit_kernel<Real, 1><<<(unsigned)((rows0 + bs - 1) / bs), bs, 0, s>>>(grids, jobs, tabs);
