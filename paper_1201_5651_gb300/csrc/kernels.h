@@ -50,6 +50,7 @@ template <typename Real> struct MarchParams {
 
 // Blocks of the march: 32 x ROWS cells, NW warps of RPT rows (the measurements are in march.cuh).
 template <typename Real> struct MarchShape { enum { NW = 7, RPT = sizeof(Real) == 4 ? 3 : 1, ROWS = NW * RPT }; };
+constexpr int kMarchChunk = 8;       // layers of a trace between two progress publications
 // sets the kernel up on the current device; CTAs per SM with narr input arrays
 template <typename Real> cudaError_t march_occupancy(int narr, int *per_sm);
 template <typename Real>
@@ -100,6 +101,10 @@ OOTS_HOSTDEV inline bool make_march(March &M, int nx, int ny, int nz, const int 
 // blocks of a pyramid along u and w
 OOTS_HOSTDEV inline int march_nt1(const March &M) { return ((M.eu < M.len ? M.eu : M.len) + 31) / 32; }
 OOTS_HOSTDEV inline int march_nt2(const March &M, int rows) { return ((M.ew < M.len ? M.ew : M.len) + rows - 1) / rows; }
+// Layers an item publishes: [first, len) of its pyramid, first = its l0.  A chunk is staged whole, also
+// where its first layers lie before the neighbour's and its last ones beyond the pyramid: those are no
+// cells of the halo.
+OOTS_HOSTDEV inline bool march_published(int l, int first, int len) { return l >= first && l < len; }
 // block (T1, T2) without its neighbours' item numbers and halo; returns the cells it publishes
 OOTS_HOSTDEV inline long long make_march_item(MarchItem &I, const March &M, int march, int T1, int T2, int rows)
 {

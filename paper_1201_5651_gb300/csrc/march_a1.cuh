@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kMarchA1Warps * 32 + 32, 1) march_a1_kernel(Ma
         const March M = P.marches[it.march];
         const GridDev<Real> &G = P.grids[M.grid];
         const int c0 = it.l0 / kA1Chunk, c1 = (M.len - 1) / kA1Chunk;
-        if (tid >= L::NC) march_hand<Real, NW, 1, kA1Chunk>(P, it, (int)tk, c0, c1, 0, epoch, phase, S);
+        if (tid >= L::NC) march_hand<Real, NW, 1, kA1Chunk>(P, it, (int)tk, c0, c1, 0, M.len, epoch, phase, S);
         else march_a1_item<Real, NW>(P, it, M, G, c0, c1, phase, S);
         if (tid == L::NC) S.next = atomicAdd(P.ticket, 1u);
         __syncthreads();
