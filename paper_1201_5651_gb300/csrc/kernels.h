@@ -1,6 +1,7 @@
 // Kernel launch interfaces used by the host driver.
 #pragma once
 #include <cuda_runtime.h>
+#include <limits.h>
 #include "oots_internal.h"
 
 #ifdef __CUDACC__
@@ -42,6 +43,7 @@ template <typename Real> struct MarchParams {
     unsigned long long *progress;      // per item: chunks of layers published, tagged with the launch's epoch
     int *err;                          // sticky device error
     long long spin_limit;              // bounded wait on upstream items
+    long long ready_limit;             // and on the CTA's own handing warp (march_ready_limit)
     long long skip_publish;            // item that never publishes (fault-injection test), -1: none
     int ngrid;                         // grids in `grids` (> 0: the launch returns at once when every
                                        // grid has reached its end time; 0: no such check)
@@ -51,6 +53,15 @@ template <typename Real> struct MarchParams {
 // Blocks of the march: 32 x ROWS cells, NW warps of RPT rows (the measurements are in march.cuh).
 template <typename Real> struct MarchShape { enum { NW = 7, RPT = sizeof(Real) == 4 ? 3 : 1, ROWS = NW * RPT }; };
 constexpr int kMarchChunk = 8;       // layers of a trace between two progress publications
+// Limits of the waits inside a CTA of the march.  The handing warp waits for other CTAs (spin_limit polls)
+// and gives up alone: what its computing warps wait for comes after that at the latest, so their limit, in
+// tests of at least ten nanoseconds, lies a thousand times its polls of about half a microsecond above it.
+// A chunk of layers takes milliseconds at most (A1: of front cells in FP64), the limit on it is a second or more.
+OOTS_HOSTDEV inline long long march_ready_limit(long long spin_limit)
+{
+    return spin_limit < ((LLONG_MAX - (1 << 24)) >> 10) ? (spin_limit << 10) + (1 << 24) : LLONG_MAX;
+}
+constexpr int kMarchDoneLimit = 1 << 24;
 // sets the kernel up on the current device; CTAs per SM with narr input arrays
 template <typename Real> cudaError_t march_occupancy(int narr, int *per_sm);
 template <typename Real>

@@ -116,9 +116,7 @@ __device__ __forceinline__ void march_a1_item(const MarchParams<Real> &P, const 
     double ions = 0.0, rec = 0.0;
     for (int c = c0; c <= c1; c++, phase++) {
         const int b = (int)(phase & 1u);
-        long long spins = 0;
-        while (!mb_test(&S.ready[b], (phase >> 1) & 1u))
-            if (++spins > (P.spin_limit << 4)) { atomicCAS(P.err, 0, (int)DEVERR_TIMEOUT); break; }
+        march_await(P, S, phase);
         for (int q = 0; q < H; q++, g += sl, phalo += L::STRIDE) {
             const int l = c * H + q;
             if (l < l0 || l >= len) continue;
@@ -220,6 +218,7 @@ __global__ void __launch_bounds__(kMarchA1Warps * 32 + 32, 1) march_a1_kernel(Ma
         else march_a1_item<Real, NW>(P, it, M, G, c0, c1, phase, S);
         if (tid == L::NC) S.next = atomicAdd(P.ticket, 1u);
         __syncthreads();
+        march_item_end(S, phase);
     }
     march_end(P, epoch);
 }

@@ -218,6 +218,7 @@ int trace_noalloc(DevSetup &S, int nx, int ny, int nz, double dx, const void *n_
     P.progress = progress;
     P.err = (int *)(sc + kOffErr);
     P.spin_limit = 1ll << 22;
+    P.ready_limit = march_ready_limit(P.spin_limit);
     P.skip_publish = -1;
     P.ngrid = 0;
     P.narr = narr;

@@ -490,6 +490,7 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
         P.progress = L.progress;
         P.err = d_err;
         P.spin_limit = spin_limit;
+        P.ready_limit = march_ready_limit(spin_limit);
         P.skip_publish = skip_publish;
         P.ngrid = (int)ctxs.size();
         P.narr = narr;

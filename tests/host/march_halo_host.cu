@@ -49,3 +49,6 @@ extern "C" void oots_host_march_halo(int nx, int ny, int nz, const int *v, int r
             }
         }
 }
+
+// the computing warps' limit on their wait for the halo (kernels.h)
+extern "C" long long oots_host_march_ready_limit(long long spin_limit) { return march_ready_limit(spin_limit); }

@@ -44,3 +44,13 @@ def test_staged_halo_lies_in_the_neighbours_cells(lib, rows, chunk, sectors):
         assert (out[1], out[2]) == (0, 0), (n, v, list(out))
         staged += out[0]
     assert staged > 10 ** 6
+
+
+def test_limit_on_the_halo_lies_above_the_limit_on_other_blocks(lib):
+    """The handing warp alone gives up on other blocks: its CTA's own limit is a multiple of that limit for
+    every limit that can be set, up to the largest (a product that overflowed gave up at the first test)."""
+    lib.oots_host_march_ready_limit.restype = ctypes.c_longlong
+    lib.oots_host_march_ready_limit.argtypes = [ctypes.c_longlong]
+    top = 2 ** 63 - 1
+    for s in [1, 2, 2000, 1 << 22, 1 << 40, 1 << 53, 1 << 59, 1 << 60, 1 << 62, top]:
+        assert lib.oots_host_march_ready_limit(s) >= min(1024 * s, top), s
