@@ -197,8 +197,9 @@ template <> struct IntCfg<double> {
     static OOTS_HD double umax() { return 40.0; }
     static OOTS_HD double tolq() { return 1e-14; }
     static OOTS_HD double zlin() { return 1e-6; }    // linearised step allowed below this h|f'|
-    // series step: terms, largest h|f'| (z^9/9! is 3e-15 there) and largest change in units of the bending
-    // scale 1/b (the cubic through both ends is then off by delta^4/384 = 7e-13 of f)
+    // series step: terms, largest h|f'| (what e^z leaves out is then z^8/8! = 4e-14 of the change; the terms
+    // left out are checked in the step itself) and largest change in units of the bending scale 1/b (the
+    // cubic through both ends is then off by delta^4/384 = 7e-13 of f)
     enum { KSER = 8 };
     static OOTS_HD double zser() { return 0.08; }
     static OOTS_HD double dser() { return 4e-3; }
@@ -408,8 +409,11 @@ OOTS_HD bool near_root_solution(const CellODE<Real> &C, Real xe, Real d0, Real D
 // and the solution of dx/dt = cubic is its power series in t, whose
 // coefficients follow from one another by Cauchy products.  One evaluation of
 // the rates; the quadrature spends 24 and more, and before this form took nine
-// in ten of the cells that the FP64 path queued.  bm: largest 1/scale; returns
-// false when the cell is not that slow.
+// in ten of the cells that the FP64 path queued.  The recombination term bends
+// on no scale of bm and, near x = 1, hardly shows in f': what the series leaves
+// out is judged by its own last terms (coefficients fall by at most rho = |a1|
+// + sqrt|a0 a2| from one to the next), against a quarter of the rounding of x.
+// bm: largest 1/scale; returns false when the cell is not that slow.
 template <typename Real, int NSMAX>
 OOTS_HD bool series_step(const CellODE<Real> &C, Real x0, Real h, Real f0, Real df0, Real bm, IntResult<Real> &R)
 {
@@ -441,6 +445,8 @@ OOTS_HD bool series_step(const CellODE<Real> &C, Real x0, Real h, Real f0, Real 
         }
         S[k + 1] = (a1 * S[k] + a2 * Q[k] + a3 * T[k]) * (Real(1) / Real(k + 1));
     }
+    const Real rho = m_abs(a1) + m_sqrt(m_abs(a2 * a0));
+    if (!(rho <= Real(0.5) && ad * rho * (m_abs(S[K]) + rho * m_abs(S[K - 1])) <= Real(0.25) * RealLimits<Real>::eps() * x0)) return false;
     Q[K] = Real(0);
 #pragma unroll
     for (int i = 1; i < K; i++) Q[K] += S[i] * S[K - i];
