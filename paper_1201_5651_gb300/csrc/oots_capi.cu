@@ -658,13 +658,15 @@ static int check_ctx(const oots_ctx *c)
 // place of 6.1.)
 __global__ void push_state_kernel(DevState *st, const __grid_constant__ DevState v) { *st = v; }
 
+// (A batch's work runs on the batch's stream, which these do not wait for: of a context in a batch only
+// batch_pull knows the state.)
 static int pull_state(oots_ctx *c)
 {
     CU(cudaSetDevice(c->device));
     CU(cudaMemcpyAsync(&c->rb->st, c->d_st, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
     c->h_st = c->rb->st;
-    c->st_current = true;
+    c->st_current = !c->batched;
     return OOTS_OK;
 }
 
@@ -673,7 +675,7 @@ static int push_state(oots_ctx *c)
     CU(cudaSetDevice(c->device));
     push_state_kernel<<<1, 1, 0, c->stream>>>(c->d_st, c->h_st);
     CU(cudaGetLastError());
-    c->st_current = true;
+    c->st_current = !c->batched;
     return OOTS_OK;
 }
 
@@ -1660,7 +1662,10 @@ int oots_batch_destroy(oots_batch *b)
         cudaSetDevice(b->ctxs[0]->device);
         cudaStreamSynchronize(b->stream);
     }
-    for (auto *c : b->ctxs) c->batched = false;
+    for (auto *c : b->ctxs) {
+        c->batched = false;
+        c->st_current = false;
+    }
     delete b;
     return OOTS_OK;
 }
