@@ -229,13 +229,19 @@ OOTS_HD Real attenuation_average(const CellODE<Real> &C, const SrcEq<Real> *Q, R
 // monotonically to it.  f is a difference of two terms, so it is known only to
 // about eps times their size: Newton also stops once |f| is inside that
 // rounding band (the iterate would otherwise jitter inside it without meeting
-// the step test).
+// the step test).  The band is some ten times the true rounding of f, so the
+// step from there is still taken: it costs no evaluation, and without it a root
+// could be off by 32 eps (1 - x), which a step of several relaxation times
+// passes on to x.
 template <typename Real, int NSMAX>
 OOTS_HD Real newton_root(const CellODE<Real> &C, Real lo, Real hi, Real xk, Real fk, Real Fk, Real dfk)
 {
     Real xe = xk;
     for (int it = 0; it < 60; it++) {
-        if (m_abs(fk) <= Real(32) * RealLimits<Real>::eps() * (m_abs(Fk) + C.c * (Real(1) - xk) * (Real(1) - xk))) break;
+        if (m_abs(fk) <= Real(32) * RealLimits<Real>::eps() * (m_abs(Fk) + C.c * (Real(1) - xk) * (Real(1) - xk))) {
+            if (dfk < Real(0)) xe = m_min(m_max(xk - fk / dfk, lo), hi);
+            break;
+        }
         if (fk > Real(0)) lo = m_max(lo, xk); else hi = m_min(hi, xk);
         Real xn = (dfk < Real(0)) ? xk - fk / dfk : Real(0.5) * (lo + hi);
         if (!(xn >= lo && xn <= hi)) xn = Real(0.5) * (lo + hi);
@@ -578,6 +584,7 @@ OOTS_HD bool integrate_prelude(const CellODE<Real> &C, Real x0, Real h, Real sig
             fk = -Fk + C.c * (Real(1) - xk) * (Real(1) - xk);
             dfk = -dFk - Real(2) * C.c * (Real(1) - xk);
             if (m_abs(fk) <= Real(32) * RealLimits<Real>::eps() * (m_abs(Fk) + C.c * (Real(1) - xk) * (Real(1) - xk))) {
+                if (dfk < Real(0)) xk = m_min(m_max(xk - fk / dfk, Real(0)), Real(1));
                 conv = true;
                 break;
             }
