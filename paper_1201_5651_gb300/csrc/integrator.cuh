@@ -204,8 +204,9 @@ template <> struct IntCfg<double> {
     static OOTS_HD double zser() { return 0.08; }
     static OOTS_HD double dser() { return 4e-3; }
     // near the root: largest b |x0 - x_eq| when the step relaxes it by e^-45, and at all with A1's average
+    // (which is then off by its square, as the quadrature is)
     static OOTS_HD double drel() { return 4e-3; }
-    static OOTS_HD double davg() { return 1e-6; }
+    static OOTS_HD double davg() { return 3e-7; }
 };
 template <> struct IntCfg<float> {
     enum { G = 4 };
@@ -385,11 +386,14 @@ OOTS_HD void root_slope(const CellODE<Real> &C, Real xe, Real sigma0, SrcEq<Real
 
 // Already next to the root (|d0| = |x0 - x_eq| far below both bending scales):
 // the linearised solution about x_eq, d(t) = d0 e^{-Dinf t}.  A step that
-// relaxes the deviation by e^-45 leaves x = x_eq whatever its path, which only
-// the small time integrals see, so the deviation may be larger there.  Returns
-// false when the state is not that close.
+// relaxes the deviation by e^-45 leaves x = x_eq whatever its path, so the
+// deviation may be larger there; the recombinations then come from the time as
+// an integral over d, dt = -dd / (d D), whose secant slope D(d) is known at
+// both ends, and its slope at d0, from f0 = f(x0) and df0 = f'(x0) (an error of
+// (b d0)^3 / 300 of a term that is itself below d0/45 of them).  Returns false
+// when the state is not that close.
 template <typename Real>
-OOTS_HD bool near_root_solution(const CellODE<Real> &C, Real xe, Real d0, Real Dinf, Real bmax, Real h,
+OOTS_HD bool near_root_solution(const CellODE<Real> &C, Real xe, Real d0, Real Dinf, Real bmax, Real h, Real f0, Real df0,
                                 IntResult<Real> &R)
 {
     const Real ad0 = m_abs(d0), one = Real(1) - xe, q = Dinf * h;
@@ -401,6 +405,15 @@ OOTS_HD bool near_root_solution(const CellODE<Real> &C, Real xe, Real d0, Real D
     const Real g1 = (q > Real(1e-6)) ? -m_expm1(-q) / Dinf : h;
     const Real g2 = (q > Real(1e-6)) ? -m_expm1(Real(-2) * q) / (Real(2) * Dinf) : h;
     R.IR = C.c * (one * one * h - Real(2) * one * d0 * g1 + d0 * d0 * g2);
+    if (C.b0 == Real(0) && q > Real(45) && ad0 > Real(0)) {
+        const Real D1 = -f0 / d0, dD = D1 - Dinf;
+        if (m_abs(dD) <= Real(0.1) * Dinf) {         // (not so: f0 is rounding alone, and d0 too small to matter)
+            // D at the middle from both ends and d0 D'(d0) = -df0 - D1; Simpson's rule
+            const Real Dm = Dinf + Real(0.75) * dD + Real(0.25) * (df0 + D1);
+            const Real J = (Real(-2) * one) / Dinf + Real(4) * (Real(0.5) * d0 - Real(2) * one) / Dm + (d0 - Real(2) * one) / D1;
+            R.IR = C.c * (one * one * h + d0 * J * (Real(1) / Real(6)));
+        }
+    }
     if (C.b0 > Real(0)) {
         // mean of exp(-b0 (xe + d)), b0 d at most davg
         const Real y = C.b0 * d0;
@@ -591,7 +604,7 @@ OOTS_HD bool integrate_prelude(const CellODE<Real> &C, Real x0, Real h, Real sig
         }
         if (conv) {
             // the slope at the root is the last one of the Newton steps
-            if (near_root_solution<Real>(C, xk, x0 - xk, -dfk, bm, h, R)) return true;
+            if (near_root_solution<Real>(C, xk, x0 - xk, -dfk, bm, h, f0, df0, R)) return true;
             R.x = x0;          // not close enough: leave it to the general part
             R.IR = Real(0);
         }
@@ -619,7 +632,7 @@ OOTS_HD IntResult<Real> integrate_general(const CellODE<Real> &C, Real x0, Real 
     Real Dinf, bmax;
     root_slope<Real, NSMAX>(C, xe, sigma0, Q, Dinf, bmax);
     const Real ad0 = m_abs(d0);
-    if (near_root_solution<Real>(C, xe, d0, Dinf, bmax, h, R)) return R;
+    if (near_root_solution<Real>(C, xe, d0, Dinf, bmax, h, f0, -dF0 - Real(2) * C.c * (Real(1) - x0), R)) return R;
     // start of the near-equilibrium tail in w = e^u: the secant slope bends on
     // |d| ~ 1/bmax (photoionisation) and |d| ~ 1 - xe (recombination)
     Real wt = Real(1);
