@@ -124,7 +124,7 @@ __device__ __forceinline__ void march_a1_item(const MarchParams<Real> &P, const 
             const Real n = act ? (nd ? __ldg(nd + g) : nu) : Real(1), x0 = act ? __ldg(xs + g) : Real(1);
             // entry column: the neighbours and weights of march_item
             const bool e1 = u >= l, e2 = w >= l;
-            const Real ica = mr_rcp(Real(2 * l + 1));
+            const Real ica = Real(1) / Real(2 * l + 1);
             const Real g1 = e1 ? Real(1) : Real(2 * u + 1) * ica, g2 = e2 ? Real(1) : Real(2 * w + 1) * ica;
             const Real p1 = Real(1) - g1, p2 = Real(1) - g2;
             const MCell<Real> bel = warp > 0 ? S.row[(l + 1) & 1][warp > 0 ? warp - 1 : 0][lane] : S.bot[b][q][lane + 1];
