@@ -326,17 +326,20 @@ __global__ void __launch_bounds__(BS, (sizeof(Real) == 4 ? 1024 : 512) / BS) cel
 // thread (cell_seq_kernel) instead of a lane group.  By the grid's own count,
 // so that a grid takes the same path, and the same rounding, in any batch.
 // Measured in FP32, lane groups against threads (us): 16 k cells 69 / 170,
-// 46 k 92 / 115, 112 k 313 / 170, 162 k with many sources 1283 / 381.  In FP64
-// groups win at 9 k cells (2.9 ms / 5.5 ms: few warps, and a warp waits for
-// the longest of its cells in every loop) and no measured queue is longer.
-template <typename Real> __host__ __device__ constexpr unsigned seq_cells() { return 65536u; }
+// 46 k 92 / 115, 112 k 313 / 170, 162 k with many sources 1283 / 381.  In FP64,
+// blackbody sources (ms), one source: 8 k cells 2.4 / 4.7, 20 k 5.8 / 6.3, 60 k
+// 16.1 / 10.0, 128 k 33 / 19, 400 k 107 / 47; three sources: 8 k 5.4 / 15.4,
+// 22 k 14.2 / 22.5, 64 k 39.9 / 27.1, 141 k 91 / 60, 512 k 314 / 180.  (Few
+// cells leave most threads idle, and a warp waits for the longest of its cells
+// in every loop.)  The lines lie where threads are no slower in either.
+template <typename Real> __host__ __device__ constexpr unsigned seq_cells() { return sizeof(Real) == 4 ? 65536u : 40960u; }
 
 // General pass: one lane group per queued cell (a half warp in FP32, a warp
 // in FP64; HALF: queue 0, FULL: queue 1).  Groups take the next queued cell
 // from a head counter (qcount[2 + queue]), so the pass ends when the cells
 // run out rather than when the group that drew the slowest share finishes.
 // Every lane forms the same rates and runs the same root search; the
-// quadrature nodes are spread over the lanes (WarpEval).  Budget sums of FULL
+// quadrature nodes are spread over the lanes (GroupEval).  Budget sums of FULL
 // are gathered per block in shared memory for up to eight grids and flushed
 // with one atomic per grid and block.
 template <typename Real, int OP>
