@@ -33,7 +33,7 @@ constexpr int kMaxItems = 4096;                 // blocks of all pyramids (a gri
 constexpr int kMaxItemDiag = 2048;              // block diagonals T1 + T2 of a pyramid (sides up to 8192)
 
 // header layout (byte offsets inside the scratch)
-constexpr size_t kOffTicket = 0;                // ticket, then the count of finished CTAs (each launch leaves them zero)
+constexpr size_t kOffTicket = 0;                // ticket, then the count of finished CTAs
 constexpr size_t kOffEpoch = 64;                // marches so far: never cleared (progress words carry it)
 constexpr size_t kOffErr = 128;
 constexpr size_t kOffState = 256;               // DevState (done = 0 after the clear)
@@ -79,6 +79,9 @@ __global__ void build_worklist(const __grid_constant__ MarchSet S, const __grid_
         s_halo = 0u;
         *(GridDev<Real> *)(sc + kOffGrid) = G0;
         *(int *)(sc + kOffErr) = 0;
+        // (a launch leaves these zero, but one cut across by another call may not have)
+        ((unsigned *)(sc + kOffTicket))[0] = 0u;
+        ((unsigned *)(sc + kOffTicket))[1] = 0u;
         DevState *st = (DevState *)(sc + kOffState);
         st->done = 0;
     }
