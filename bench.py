@@ -256,14 +256,12 @@ def step_bytes_per_cell(nsrc, n_array):
     return 28 * nsrc + 32
 
 
-def _describe_tile(shape, cell_block=None, nsrc=1):
-    """The tile shape asked for and the trace kernel, and (when given) the threads per block of
-    the closed-form per-cell passes (0 = the library's default for the source count)."""
-    from paper_1201_5651_gb300 import oots
+def _describe_tile(shape, cell_block=None, nsrc=1, rows=21):
+    """The trace kernel and its block (32 x 21 cells; FP64 32 x 7), and (when given) the threads per
+    block of the closed-form per-cell passes (0 = the library's default for the source count)."""
     if shape is None:
         return None
-    dims = oots.oots_tile_shape_info(shape)[1]
-    d = {"id": shape, "dims": list(dims), "kernel": "march"}
+    d = {"kernel": "march", "block": [32, rows]}
     if cell_block is not None:
         d["cell_block"] = cell_block if cell_block else (128 if nsrc > 1 else 256)
     return d
@@ -336,7 +334,7 @@ def _timed_substeps(run_one, sync, stream, flush, steps, warmup):
 
 
 def _tuned_context(w, precision, dev, stream, args, devname):
-    """A context on `stream`, its tile shape chosen by the autotuner at t = 0 (the
+    """A context on `stream`, its per-cell block size chosen by the autotuner at t = 0 (the
     tuning substeps are then undone: state, time and budget reset)."""
     from paper_1201_5651_gb300 import autotune, oots
     c = oots.Context.from_workload(w, precision, device=dev, scheme=oots.OOTS_A3, K4=0.25)
@@ -429,7 +427,7 @@ def bench_single(args, name, steps, warmup, rank, world, dev, flush, devname, wi
         xm = cm.get_neutral_fraction()
         rm, rf = _reff(xm, w.dx, spec["n_oct"]), _reff(xf, w.dx, spec["n_oct"])
         out["fp64"] = {"value": job_rate(w.ncell * k64, world, ms64), "ms_per_step": ms64 / k64, "steps": k64,
-                       "warmup": 1, "tile_shape": _describe_tile(shape)}
+                       "warmup": 1, "tile_shape": _describe_tile(shape, rows=7)}
         out["mixed_over_fp64"] = value / out["fp64"]["value"]
         out["accuracy_vs_fp64"] = {
             "from_t_over_trec": t0 / trec, "t_over_trec": tf / trec, "fp64_substeps": k64 + 1,
@@ -679,7 +677,7 @@ def main():
     ap.add_argument("--workload", default="multisource512_bb", choices=sorted(WORKLOADS))
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-extra-configs", action="store_true", help="skip the 256^3 and 64-grid lines")
-    ap.add_argument("--shape", type=int, default=-1, help="tile shape id (-1: autotuned)")
+    ap.add_argument("--shape", type=int, default=-1, help="tile shape id, checked and kept (-1: the autotuner's)")
     ap.add_argument("--retune", action="store_true", help="ignore the autotuner cache")
     args = ap.parse_args()
     world = int(os.environ.get("WORLD_SIZE", "1"))

@@ -1,18 +1,18 @@
-"""Autotuner for a substep's launch shapes: the trace's tile shape and the
-block size of the closed-form per-cell passes.
+"""Autotuner for the block size of the closed-form per-cell passes (the dt
+criterion, the half and the full step).
+
+Small blocks hold up fewer cells behind a slow one at their barriers, large
+ones set up fewer blocks; which wins depends on how uneven the per-cell work is
+(many sources, fronts).  The tuner keys its choice on a plane-size class of the
+launch -- the largest grid side (rounded up to a power of two), the number of
+sources per grid and the number of grids, each bucketed -- rather than on the
+exact grid, times both sizes on one substep (per-launch CUDA events through
+oots_profile_substep, or whole batched substeps), and caches the faster as JSON
+keyed by device name, precision and class.
 
 The trace runs one block shape per precision whatever tile shape is asked for,
-so the shapes differ by noise now; the interface and the cache keep them.  The
-tuner keys its choice on a plane-size class of the launch -- the largest grid side (rounded up to a
-power of two), the number of sources per grid and the number of grids, each
-bucketed -- rather than on the exact grid, times every shape the device can
-run on one substep (per-launch CUDA events through oots_profile_substep, or
-whole batched substeps), and caches the fastest as JSON keyed by device name,
-precision and class.  On the chosen shape it then times the closed-form
-per-cell passes (the dt criterion, the half and the full step) with 128- and
-256-thread blocks: small blocks hold up fewer cells behind a slow one at their
-barriers, large ones set up fewer blocks, and which wins depends on how
-uneven the per-cell work is (many sources, fronts).
+so no tile shape is timed: an entry holds TILE_SHAPE, and a cached entry's shape
+is still handed to the context.
 """
 from __future__ import annotations
 
@@ -79,6 +79,7 @@ def lookup_cell_block(device_name: str, precision: int, klass: str, path: str = 
 
 CELL_KINDS = ("ratedt", "ratedt_verify", "half", "full")
 CELL_BLOCKS = (128, 256)
+TILE_SHAPE = 0
 
 
 def _tune_cell_block(ctx: "oots.Context", repeats: int) -> Dict[int, float]:
@@ -98,15 +99,10 @@ def _tune_cell_block(ctx: "oots.Context", repeats: int) -> Dict[int, float]:
     return times
 
 
-def _shapes():
-    n, _ = oots.oots_tile_shape_info(0)
-    return range(n)
-
-
 def tune(ctx: "oots.Context", device_name: str, nsrc: int, repeats: int = 2, use_cache: bool = True,
          verbose: bool = False, path: str = CACHE) -> Optional[int]:
-    """Time every tile shape on ctx (which it advances by a few substeps) and
-    select the fastest for the sweep; returns the chosen shape."""
+    """Time the per-cell passes' block sizes on ctx (which it advances by a few
+    substeps) and set the faster; returns the tile shape (TILE_SHAPE, or a cached entry's)."""
     nz, ny, nx = ctx.shape
     klass = plane_class(nx, ny, nz, nsrc)
     key = cache_key(device_name, ctx.precision, klass)
@@ -118,42 +114,22 @@ def tune(ctx: "oots.Context", device_name: str, nsrc: int, repeats: int = 2, use
             if cb:
                 ctx.set_cell_block(cb)
             return hit
-    times = {}
-    for sh in _shapes():
-        try:
-            ctx.set_tile_shape(sh)
-            ctx.profile_substep()                     # build + warm up this shape
-            best = None
-            for _ in range(repeats):
-                prof = dict()
-                for k, ms in ctx.profile_substep():
-                    prof[k] = prof.get(k, 0.0) + ms
-                t = sum(v for k, v in prof.items() if k.startswith("sweep"))
-                best = t if best is None else min(best, t)
-            times[sh] = best
-        except oots.OotsError:
-            continue                                  # shape does not fit at this precision
-    if not times:
-        return None
-    choice = min(times, key=times.get)
-    ctx.set_tile_shape(choice)
+    ctx.set_tile_shape(TILE_SHAPE)
     ctimes = _tune_cell_block(ctx, repeats)
     cb = min(ctimes, key=ctimes.get) if ctimes else 0
     ctx.set_cell_block(cb)
     if verbose:
-        print({sh: round(v, 4) for sh, v in times.items()}, {b: round(v, 4) for b, v in ctimes.items()})
-    _store(key, {"shape": choice, "dims": oots.oots_tile_shape_info(choice)[1], "class": klass,
-                 "sweep_ms": {str(k): v for k, v in times.items()}, "cell_block": cb,
+        print({b: round(v, 4) for b, v in ctimes.items()})
+    _store(key, {"shape": TILE_SHAPE, "class": klass, "cell_block": cb,
                  "cell_ms": {str(k): v for k, v in ctimes.items()}}, path)
-    return choice
+    return TILE_SHAPE
 
 
 def tune_batch(ctxs: Sequence["oots.Context"], workloads, device_name: str, repeats: int = 2,
                use_cache: bool = True, path: str = CACHE) -> Optional[int]:
-    """Time whole batched substeps of the contexts for every tile shape, then
-    for each block size of the closed-form passes on the fastest shape; keep
-    the fastest of each (the block size is set on the contexts, the shape
-    returned).  The contexts' states and times are restored afterwards."""
+    """Time whole batched substeps of the contexts for each block size of the
+    closed-form passes and set the faster on the contexts; returns the tile
+    shape, as tune does.  The contexts' states and times are restored afterwards."""
     nside = max(max(w.nx, w.ny, w.nz) for w in workloads)
     nsrc = max(len(w.sources) for w in workloads)
     klass = plane_class(nside, nside, nside, nsrc, len(ctxs))
@@ -169,9 +145,9 @@ def tune_batch(ctxs: Sequence["oots.Context"], workloads, device_name: str, repe
             return hit
     t_end = [10.0 * w.t_rec for w in workloads]
 
-    def timed(sh, cb):
+    def timed(cb):
         for c in ctxs:
-            c.set_tile_shape(sh)
+            c.set_tile_shape(TILE_SHAPE)
             c.set_cell_block(cb)
         b = oots.Batch(ctxs)
         try:
@@ -188,28 +164,18 @@ def tune_batch(ctxs: Sequence["oots.Context"], workloads, device_name: str, repe
         finally:
             b.close()
 
-    times, ctimes = {}, {}
-    for sh in _shapes():
+    ctimes = {}
+    for cb in CELL_BLOCKS:
         try:
-            times[sh] = timed(sh, 0)
+            ctimes[cb] = timed(cb)
         except oots.OotsError:
             continue
-    choice = min(times, key=times.get) if times else None
-    if choice is not None:
-        for cb in CELL_BLOCKS:
-            try:
-                ctimes[cb] = timed(choice, cb)
-            except oots.OotsError:
-                continue
     cb = min(ctimes, key=ctimes.get) if ctimes else 0
     for c, w in zip(ctxs, workloads):
         c.set_cell_block(cb)
         c.set_neutral_fraction(w.x0)
         c.set_time(0.0)
         c.reset_budget()
-    if choice is None:
-        return None
-    _store(key, {"shape": choice, "dims": oots.oots_tile_shape_info(choice)[1], "class": klass,
-                 "substep_ms": {str(k): v for k, v in times.items()}, "cell_block": cb,
+    _store(key, {"shape": TILE_SHAPE, "class": klass, "cell_block": cb,
                  "cell_substep_ms": {str(k): v for k, v in ctimes.items()}}, path)
-    return choice
+    return TILE_SHAPE
