@@ -195,8 +195,8 @@ int oots_run_substeps(oots_ctx *ctx, long long n, double t_end);
 #define OOTS_K_FULL      6   /* full-step integration and photon budget  */
 #define OOTS_K_FINAL1    7   /* close the substep                        */
 #define OOTS_K_IMPLICIT  8   /* implicit sweep (A1)                      */
-#define OOTS_K_HALF_GENERAL 9  /* half step, cells no closed form settles (one warp each) */
-#define OOTS_K_FULL_GENERAL 10 /* full step, cells no closed form settles (one warp each) */
+#define OOTS_K_HALF_GENERAL 9  /* half step, cells no closed form settles (a lane group or a thread each) */
+#define OOTS_K_FULL_GENERAL 10 /* full step, cells no closed form settles (a lane group or a thread each) */
 #define OOTS_K_PLANE_TRACE 11  /* columns of the plane-parallel sources (either trace) */
 #define OOTS_K_PLANE_IMPLICIT 12 /* A1 row integration of a plane-parallel source */
 #define OOTS_K_PACK      13  /* n x of the traced state, packed (before a trace of several sources) */

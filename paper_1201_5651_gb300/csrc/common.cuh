@@ -57,17 +57,6 @@ OOTS_HD __forceinline__ ff ff_mul_f(ff a, float f)
     e = fmaf(a.lo, f, e);
     return ff_quick(p, e);
 }
-// a / f with one correction step (remainder computed exactly)
-OOTS_HD __forceinline__ ff ff_div_f(ff a, float f)
-{
-    float q1 = a.hi / f;
-    float p = q1 * f;
-    float pe = fmaf(q1, f, -p);
-    // remainder r = a - q1 f computed as (a.hi - p) - pe + a.lo
-    float r = ((a.hi - p) - pe) + a.lo;
-    float q2 = r / f;
-    return ff_quick(q1, q2);
-}
 
 // Column type per precision: FP64 path carries double, mixed path float-float.
 template <typename Real> struct ColT;
@@ -75,28 +64,20 @@ template <> struct ColT<double> {
     typedef double type;
     static OOTS_HD __forceinline__ double zero() { return 0.0; }
     static OOTS_HD __forceinline__ double fma_w(double acc, double w, double N) { return fma(w, N, acc); }
-    static OOTS_HD __forceinline__ double div(double a, double s) { return a / s; }
     static OOTS_HD __forceinline__ double add(double a, double d) { return a + d; }
     static OOTS_HD __forceinline__ double addc(double a, double b) { return a + b; }
     static OOTS_HD __forceinline__ double to_real(double a) { return a; }
     static OOTS_HD __forceinline__ double sub_r(double a, double b) { return a - b; }
-    static OOTS_HD __forceinline__ double make(double hi, double) { return hi; }
-    static OOTS_HD __forceinline__ double hi(double a) { return a; }
-    static OOTS_HD __forceinline__ double lo(double) { return 0.0; }
 };
 template <> struct ColT<float> {
     typedef ff type;
     static OOTS_HD __forceinline__ ff zero() { return ff{0.0f, 0.0f}; }
     static OOTS_HD __forceinline__ ff fma_w(ff acc, float w, ff N) { return ff_add(acc, ff_mul_f(N, w)); }
-    static OOTS_HD __forceinline__ ff div(ff a, float s) { return ff_div_f(a, s); }
     static OOTS_HD __forceinline__ ff add(ff a, float d) { return ff_add_f(a, d); }
     static OOTS_HD __forceinline__ ff addc(ff a, ff b) { return ff_add(a, b); }
     static OOTS_HD __forceinline__ float to_real(ff a) { return a.hi + a.lo; }
     // a - b rounded to one float (exact high-part difference for close columns)
     static OOTS_HD __forceinline__ float sub_r(ff a, ff b) { return (a.hi - b.hi) + (a.lo - b.lo); }
-    static OOTS_HD __forceinline__ ff make(float hi, float lo) { return ff{hi, lo}; }
-    static OOTS_HD __forceinline__ float hi(ff a) { return a.hi; }
-    static OOTS_HD __forceinline__ float lo(ff a) { return a.lo; }
 };
 
 // ---------------------------------------------------------------------------

@@ -544,7 +544,7 @@ template <typename Real> struct LaunchSet : LaunchSetBase {
             if (prof) prof->mark(OOTS_K_RATEDT_VERIFY);
             return OOTS_OK;
         }
-        // the cells no closed form settles, one warp each
+        // the cells no closed form settles: a lane group each, or in a long queue a thread
         if (prof) prof->mark(0);
         CU(launch_cell<Real>(d_grids, (int)ctxs.size(), d_offsets, total, d_tabs, op | OP_GENERAL, nsmax, d_queue,
                              d_qcount, d_qrec, d_rcache, 0, gen_blocks, cell_bs, s));
@@ -681,7 +681,7 @@ static int push_state(oots_ctx *c)
 
 static int device_error(int err)
 {
-    if (err == DEVERR_TIMEOUT) return fail(OOTS_E_DEVICE_TIMEOUT, "a wavefront tile gave up waiting for its upstream tiles");
+    if (err == DEVERR_TIMEOUT) return fail(OOTS_E_DEVICE_TIMEOUT, "a block of the trace gave up waiting for its upstream blocks");
     if (err) return fail(OOTS_E_CUDA, "device error %d", err);
     return OOTS_OK;
 }
