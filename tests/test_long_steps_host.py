@@ -37,15 +37,3 @@ def test_near_neutral_cells_over_long_steps(lib, x0):  # noqa: F811
                 assert abs(out[0] - xr) <= tol, (precision, x0, ch, b, g, b0, out[0] - xr)
                 if b0 > 0:
                     assert abs(out[2] - lr) <= tol * max(1.0, bb), (precision, x0, ch, b, g, out[2] - lr)
-
-
-@pytest.mark.parametrize("x0", [0.5, 0.9, 0.99, 0.999])
-def test_root_below_the_rounding_band_mixed(lib, x0):  # noqa: F811
-    """Cells that go to the quadrature and fall by a third: its 1e-6 of the change, a rounding of the result
-    and one of the rate over the step make 5e-7.  A root anywhere in the band in which f is taken for zero
-    (32 roundings of the rate) leaves twice that."""
-    for ch, b in itertools.product([0.1, 0.3], [1.0, 3.0]):
-        A, bb, c, x = (float(np.float32(v)) for v in (0.5 / b / H, b, ch / H, x0))
-        out = np.zeros(3)
-        lib.oots_host_integrate_mono(1, A, bb, 0.0, c, 0.0, SIG, x, H, out.ctypes.data)
-        assert abs(out[0] - _reference(A, bb, c, x)[0]) <= 5e-7, (x0, ch, b)
